@@ -89,6 +89,8 @@ _SIGS = {
 }
 
 _lib = None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def lib() -> ctypes.CDLL:
@@ -121,15 +123,26 @@ def _p(t):
 
 def _stream(stream):
     if stream is None:
+        # The current stream's handle as torch keeps it: 0.2 us, against 2.9 us
+        # for building the torch.cuda.Stream object (a third of a small call's
+        # host time on the Grace host).  Before CUDA is initialised the object's
+        # constructor initialises it.
+        if torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
 
 
+# int arrays of the usual group counts; looking the type up costs more than
+# filling it
+_INT_ARRAYS = tuple(ctypes.c_int * max(1, n) for n in range(33))
+
+
 def _host_ints(xs) -> ctypes.Array:
-    xs = list(xs)
-    return (ctypes.c_int * max(1, len(xs)))(*xs)
+    n = len(xs := tuple(xs))
+    return (_INT_ARRAYS[n] if n < len(_INT_ARRAYS) else ctypes.c_int * n)(*xs)
 
 
 def _check(st: int, where: str) -> int:
