@@ -68,6 +68,12 @@ __device__ __forceinline__ void set_error(unsigned *err, unsigned bit) {
   atomicOr(err, bit);
 }
 
+// fp32 active attention (hsa_attention_f32.cu) over checked arguments.
+int launch_attention_f32(const void *q, const int32_t *q_idx, int n_active, const void *k_cache,
+                         const void *v_cache, int rows1, const void *k_base, const void *v_base,
+                         int rows2, int H, int D, float scale, void *out, cudaStream_t stream,
+                         unsigned *err);
+
 // Number of lanes that cooperate on one row of `vecs` 16-byte vectors:
 // a power of two, at most 32.
 inline int lanes_per_row(long long vecs) {
