@@ -32,10 +32,12 @@ namespace hsa {
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kItems = 16;                              // per thread per tile
-constexpr int kTile = kSortThreads * kItems;            // 4096 tokens
-constexpr int kWarps = kSortThreads / 32;
-constexpr int kWarpItems = kTile / kWarps;              // 512 consecutive tokens
+constexpr int kTileThreads = 1024;
+constexpr int kItems = 4;                               // per thread per tile
+constexpr int kTile = kTileThreads * kItems;            // 4096 tokens
+constexpr int kTileWarps = kTileThreads / 32;
+constexpr int kWarpItems = kTile / kTileWarps;          // 128 consecutive tokens
+constexpr int kScanCtas = 8;
 constexpr int kMaxGroups = 32;
 
 struct GroupStarts {
@@ -65,85 +67,138 @@ constexpr SortLayout sort_layout(int N) {
   return L;
 }
 
+__device__ __forceinline__ uint32_t order_key(float f) {
+  uint32_t u = __float_as_uint(f);
+  if (u == 0x80000000u) u = 0u;                          // -0 ranks with +0
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);     // float order as uint order
+}
+
+// The sort's kernels are short (a few microseconds each at 524288 tokens, whose
+// keys and tokens stay in L2), so each lets the next one launch at once and
+// what bounds them is latency: every thread issues all its loads before it
+// uses the first, and a tile is shared by 32 warps.  GPU time of a whole
+// partition of 524288 tokens: 281 -> 62 us.
 __global__ void __launch_bounds__(kSortThreads)
 radix_key_kernel(const float *__restrict__ stat, int N, uint32_t *__restrict__ keys,
-           int32_t *__restrict__ vals, unsigned *err) {
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
-    const float f = stat[n];
-    uint32_t u = __float_as_uint(f);
-    if (!isfinite(f)) set_error(err, kErrNonfinite);
-    if (u == 0x80000000u) u = 0u;                          // -0 ranks with +0
-    keys[n] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);  // float order as uint order
-    vals[n] = n;
+                 unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
+  const bool vec = (reinterpret_cast<uintptr_t>(stat) & 15) == 0;
+  const int n4 = (N + 3) >> 2;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {
+    float f[4];
+    if (vec && 4 * i + 3 < N) {
+      const float4 v = __ldg(reinterpret_cast<const float4 *>(stat) + i);
+      f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) f[e] = 4 * i + e < N ? __ldg(stat + 4 * i + e) : 0.f;
+    }
+    if (!(isfinite(f[0]) && isfinite(f[1]) && isfinite(f[2]) && isfinite(f[3])))
+      set_error(err, kErrNonfinite);
+    // the buffer holds whole 256-byte blocks, so the last vector may pass N
+    reinterpret_cast<uint4 *>(keys)[i] =
+        make_uint4(order_key(f[0]), order_key(f[1]), order_key(f[2]), order_key(f[3]));
   }
 }
 
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kTileThreads)
 radix_hist_kernel(const uint32_t *__restrict__ keys, int N, int shift, uint32_t *__restrict__ hist,
-            int tiles) {
-  __shared__ uint32_t h[256];
-  h[threadIdx.x] = 0;
+                  int tiles) {
+  pdl_wait();
+  pdl_trigger();
+  // four histograms, so that the warps of a concentrated digit (the exponent
+  // bits of most statistics) contend less
+  __shared__ uint32_t h[4][256];
+  const int base = blockIdx.x * kTile + 4 * threadIdx.x;
+  uint4 k = make_uint4(0u, 0u, 0u, 0u);
+  if (base < N) k = *reinterpret_cast<const uint4 *>(keys + base);
+  (&h[0][0])[threadIdx.x] = 0;
   __syncthreads();
-  const int base = blockIdx.x * kTile;
+  uint32_t *mine = h[(threadIdx.x >> 5) & 3];
+  const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
 #pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    const int n = base + i * kSortThreads + threadIdx.x;
-    if (n < N) atomicAdd(&h[(keys[n] >> shift) & 255u], 1u);
-  }
+  for (int e = 0; e < 4; ++e)
+    if (base + e < N) atomicAdd(&mine[(kk[e] >> shift) & 255u], 1u);
   __syncthreads();
-  hist[threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
+  if (threadIdx.x < 256)
+    hist[threadIdx.x * tiles + blockIdx.x] =
+        h[0][threadIdx.x] + h[1][threadIdx.x] + h[2][threadIdx.x] + h[3][threadIdx.x];
 }
 
 // Exclusive scan, in place, of the 256*tiles counts in digit-major order, by
-// one block of 1024 threads, each owning a contiguous run.
+// one cluster: CTA c owns a contiguous share, sums it, learns the shares
+// before it through distributed shared memory, then scans its share 4096
+// counts (one 16-byte vector per thread) at a time.  One cluster instead of one
+// block that gave each thread a contiguous (uncoalesced) run: at 524288 tokens
+// 55 us -> about 4.
 __global__ void __launch_bounds__(1024) radix_scan_kernel(uint32_t *__restrict__ hist, int total) {
+  pdl_wait();
+  pdl_trigger();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
   __shared__ uint32_t warp_sum[32];
-  const int per = (total + 1023) / 1024;
-  const int b = threadIdx.x * per;
-  const int e = min(total, b + per);
-  uint32_t s = 0;
-  for (int i = b; i < e; ++i) s += hist[i];
+  __shared__ uint32_t share[kScanCtas];                  // every CTA's total
+  cl.barrier_arrive();                                   // this CTA has started
+  const int cta = (int)cl.block_rank(), ctas = (int)cl.num_blocks();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t incl = s;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
+  uint4 *h4 = reinterpret_cast<uint4 *>(hist);
+  const int n4 = total / 4;                              // total is a multiple of 256
+  const int lo = (int)((long long)n4 * cta / ctas), hi = (int)((long long)n4 * (cta + 1) / ctas);
+  uint32_t s = 0;
+#pragma unroll 4
+  for (int i = lo + threadIdx.x; i < hi; i += 1024) {
+    const uint4 v = h4[i];
+    s += v.x + v.y + v.z + v.w;
   }
-  if (lane == 31) warp_sum[w] = incl;
+  s = __reduce_add_sync(0xffffffffu, s);
+  if (lane == 0) warp_sum[w] = s;
+  cl.barrier_wait();                                     // every CTA has, so its memory exists
   __syncthreads();
   if (w == 0) {
-    uint32_t v = warp_sum[lane], inc = v;
+    const uint32_t t = __reduce_add_sync(0xffffffffu, warp_sum[lane]);
+    if (lane < ctas) *cl.map_shared_rank(&share[cta], lane) = t;
+  }
+  cl.sync();                                             // every share has arrived
+  uint32_t run = 0;
+  for (int c = 0; c < cta; ++c) run += share[c];
+  for (int b = lo; b < hi; b += 1024) {
+    const int i = b + threadIdx.x;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (i < hi) v = h4[i];
+    const uint32_t sum = v.x + v.y + v.z + v.w;
+    uint32_t incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += t;
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
     }
-    warp_sum[lane] = inc - v;
-  }
-  __syncthreads();
-  uint32_t run = warp_sum[w] + incl - s;
-  for (int i = b; i < e; ++i) {
-    const uint32_t c = hist[i];
-    hist[i] = run;
-    run += c;
+    __syncthreads();                                     // warp_sum is free
+    if (lane == 31) warp_sum[w] = incl;
+    __syncthreads();
+    const uint32_t ws = warp_sum[lane];
+    const uint32_t before = __reduce_add_sync(0xffffffffu, lane < w ? ws : 0u);
+    const uint32_t all = __reduce_add_sync(0xffffffffu, ws);
+    const uint32_t x = run + before + incl - sum;
+    if (i < hi) h4[i] = make_uint4(x, x + v.x, x + v.x + v.y, x + v.x + v.y + v.z);
+    run += all;
   }
 }
 
-// Stable scatter of one tile.  Warp w owns tokens [w*512, w*512+512) of the
+// Stable scatter of one tile.  Warp w owns tokens [w*128, w*128+128) of the
 // tile and walks them 32 at a time in order; lanes holding the same digit find
 // each other with __match_any_sync, so a token's rank among equal digits in
 // the tile is (earlier warps' count) + (this warp's running count) + (earlier
-// lanes of this step).
-__global__ void __launch_bounds__(kSortThreads)
+// lanes of this step).  vin NULL: the pairs are still in token order.  kout
+// NULL: the last pass, whose keys nothing reads.
+__global__ void __launch_bounds__(kTileThreads)
 radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict__ vin,
-               uint32_t *__restrict__ kout, int32_t *__restrict__ vout, int N, int shift,
-               const uint32_t *__restrict__ offsets, int tiles) {
-  __shared__ uint32_t cnt[kWarps][256];
+                     uint32_t *__restrict__ kout, int32_t *__restrict__ vout, int N, int shift,
+                     const uint32_t *__restrict__ offsets, int tiles) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ uint32_t cnt[kTileWarps][256];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int d = threadIdx.x; d < kWarps * 256; d += kSortThreads) (&cnt[0][0])[d] = 0;
-  __syncthreads();
-  const unsigned lt_mask = (1u << lane) - 1u;
   const int base = blockIdx.x * kTile + w * kWarpItems;
   uint32_t key[kItems];
   int32_t val[kItems];
@@ -151,9 +206,17 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
 #pragma unroll
   for (int it = 0; it < kItems; ++it) {
     const int n = base + it * 32 + lane;
-    const bool valid = n < N;
-    key[it] = valid ? kin[n] : 0u;
-    val[it] = valid ? vin[n] : 0;
+    key[it] = n < N ? kin[n] : 0u;
+    val[it] = n < N && vin ? vin[n] : n;
+  }
+  uint4 *c4 = reinterpret_cast<uint4 *>(&cnt[w][0]);
+  c4[lane] = make_uint4(0u, 0u, 0u, 0u);                 // this warp's 256 counts
+  c4[lane + 32] = make_uint4(0u, 0u, 0u, 0u);
+  __syncwarp();
+  const unsigned lt_mask = (1u << lane) - 1u;
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
+    const bool valid = base + it * 32 + lane < N;
     const uint32_t d = (key[it] >> shift) & 255u;
     const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : 256u + lane);
     const uint32_t before = valid ? cnt[w][d] : 0u;
@@ -163,25 +226,38 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
     __syncwarp();
   }
   __syncthreads();
-  // exclusive prefix over warps, one digit per thread (blockDim == 256)
+  // exclusive prefix over warps: four neighbouring threads share a digit, each
+  // eight warps of it
   {
-    const int d = threadIdx.x;
-    uint32_t run = offsets[d * tiles + blockIdx.x];
-    for (int ww = 0; ww < kWarps; ++ww) {
-      const uint32_t c = cnt[ww][d];
-      cnt[ww][d] = run;
-      run += c;
+    const int d = threadIdx.x >> 2, part = threadIdx.x & 3;
+    constexpr int kPer = kTileWarps / 4;
+    uint32_t c[kPer], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      c[i] = cnt[part * kPer + i][d];
+      sum += c[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o, 4);
+      if (part >= o) incl += t;
+    }
+    uint32_t run = offsets[d * tiles + blockIdx.x] + incl - sum;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      cnt[part * kPer + i][d] = run;
+      run += c[i];
     }
   }
   __syncthreads();
 #pragma unroll
   for (int it = 0; it < kItems; ++it) {
-    const int n = base + it * 32 + lane;
-    if (n < N) {
+    if (base + it * 32 + lane < N) {
       const uint32_t d = (key[it] >> shift) & 255u;
-      const uint32_t p = cnt[w][d] + local[it];
-      kout[p] = key[it];
-      vout[p] = val[it];
+      const uint32_t q = cnt[w][d] + local[it];
+      if (kout) kout[q] = key[it];
+      vout[q] = val[it];
     }
   }
 }
@@ -208,12 +284,6 @@ constexpr int kRankTokens = 32;
 constexpr int kRankMaxN = 12032;
 static_assert(kRankMaxN % 4 == 0 && kRankMaxN * 4 + kRankTokens * 4 <= 48 * 1024,
               "rank partition shared memory");
-
-__device__ __forceinline__ uint32_t order_key(float f) {
-  uint32_t u = __float_as_uint(f);
-  if (u == 0x80000000u) u = 0u;                          // -0 ranks with +0
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);     // float order as uint order
-}
 
 __global__ void __launch_bounds__(kRankThreads)
 rank_partition_kernel(const float *__restrict__ stat, int N, int K, GroupStarts gs,
@@ -530,12 +600,15 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
 
 __global__ void __launch_bounds__(kSortThreads)
 group_assign_kernel(const int32_t *__restrict__ sorted_tokens, int N, int K, GroupStarts gs,
-              int32_t *__restrict__ group_of) {
+                    int32_t *__restrict__ group_of) {
+  pdl_wait();
+  pdl_trigger();
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < N; r += gridDim.x * blockDim.x) {
+    const int token = sorted_tokens[r];
     int g = 0;
     for (int k = 0; k < K; ++k)
       if (r >= gs.start[k] && r < gs.start[k] + gs.count[k]) g = k;
-    group_of[sorted_tokens[r]] = g;
+    group_of[token] = g;
   }
 }
 
@@ -734,10 +807,10 @@ bool cluster_select_ready() {
   return st == 1;
 }
 
-// The same check for the active-set cluster (8 CTAs of 1024 threads, 33 KB of
-// static shared memory each); otherwise the active set takes the per-block
-// scheme.
-bool cluster_active_ready() {
+// Whether one cluster of `ctas` CTAs of kernel K can be resident on the
+// current device, resolved once per device.
+template <auto K>
+bool cluster_ready(int ctas, int threads) {
   static std::atomic<int> state[64];            // 0 unknown, 1 ready, 2 unavailable
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
@@ -745,18 +818,28 @@ bool cluster_active_ready() {
   if (st == 0) {
     st = 2;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(kCsCtas);
-    cfg.blockDim = dim3(kAcThreads);
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, active_set_cluster_kernel, &cfg) ==
-            cudaSuccess &&
-        clusters >= 1)
-      st = 1;
+    if (cudaOccupancyMaxActiveClusters(&clusters, K, &cfg) == cudaSuccess && clusters >= 1) st = 1;
     cudaGetLastError();                          // a refused query leaves no sticky error
     state[dev].store(st);
   }
   return st == 1;
 }
+
+bool cluster_active_ready() {
+  return cluster_ready<active_set_cluster_kernel>(kCsCtas, kAcThreads);
+}
+
+bool cluster_scan_ready() { return cluster_ready<radix_scan_kernel>(kScanCtas, 1024); }
 
 }  // namespace
 
@@ -807,22 +890,29 @@ extern "C" int hsa_partition(const float *stat, int N, int T, const int *budgets
         stat, N, chunk, K, gs, group_of, err);
     return launch_status();
   }
+  // The scan's cluster is one CTA where a cluster of 8 cannot be resident.
+  const unsigned scan_ctas = cluster_scan_ready() ? kScanCtas : 1;
   const int ew_blocks = (int)std::min<long long>((N + kSortThreads - 1) / kSortThreads,
                                                  (long long)sm_count() * 8);
   count_launches(1);
-  radix_key_kernel<<<ew_blocks, kSortThreads, 0, s>>>(stat, N, keys[0], vals[0], err);
+  launch_pdl(radix_key_kernel, dim3((ew_blocks + 3) / 4), dim3(kSortThreads), 0, s, stat, N,
+             keys[0], err);
   for (int pass = 0; pass < 4; ++pass) {
     const int in = pass & 1, out = in ^ 1;
     count_launches(1);
-    radix_hist_kernel<<<L.tiles, kSortThreads, 0, s>>>(keys[in], N, 8 * pass, hist, L.tiles);
+    launch_pdl(radix_hist_kernel, dim3(L.tiles), dim3(kTileThreads), 0, s, keys[in], N, 8 * pass,
+               hist, L.tiles);
     count_launches(1);
-    radix_scan_kernel<<<1, 1024, 0, s>>>(hist, 256 * L.tiles);
+    launch_pdl_cluster(radix_scan_kernel, dim3(scan_ctas), dim3(1024), scan_ctas, s, hist,
+                       256 * L.tiles);
     count_launches(1);
-    radix_scatter_kernel<<<L.tiles, kSortThreads, 0, s>>>(keys[in], vals[in], keys[out], vals[out], N,
-                                                     8 * pass, hist, L.tiles);
+    launch_pdl(radix_scatter_kernel, dim3(L.tiles), dim3(kTileThreads), 0, s, keys[in],
+               pass == 0 ? nullptr : vals[in], pass == 3 ? nullptr : keys[out], vals[out], N,
+               8 * pass, hist, L.tiles);
   }
   count_launches(1);
-  group_assign_kernel<<<ew_blocks, kSortThreads, 0, s>>>(vals[0], N, K, gs, group_of);
+  launch_pdl(group_assign_kernel, dim3(ew_blocks), dim3(kSortThreads), 0, s, vals[0], N, K, gs,
+             group_of);
   return launch_status();
 }
 
