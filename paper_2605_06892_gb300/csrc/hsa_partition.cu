@@ -16,11 +16,8 @@
 //                 order, and a stable scatter (the pairs start in token order,
 //                 so equal keys stay in token order), then rank -> group.
 //
-// The active set needs no workspace.  Up to 2097152 tokens one cluster of 8
-// CTAs marks and counts the active tokens of its ranges, exchanges the counts
-// through distributed shared memory and compacts; above that, block b owns one
-// chunk of tokens, counts the active tokens of all earlier chunks itself, then
-// compacts its own chunk with warp ballots and a block scan.
+// The active set needs no workspace: the CTAs of clusters count what comes
+// before their tokens and compact (see active_set_kernel).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -612,164 +609,154 @@ group_assign_kernel(const int32_t *__restrict__ sorted_tokens, int N, int K, Gro
   }
 }
 
-// ------------------------------------------------------------- active set
+// --------------------------------------- active set and token reordering
+//
+// Workspace-free compaction in one launch of any size: the active set lists
+// the tokens of the groups that are active; the reordering (Sec. 2.5: new
+// position r holds old token order[r]) lists the non-baseline tokens, then the
+// baseline group, each in token order.  CTA b owns `rounds` * kAcThreads *
+// kItems consecutive tokens; in a round a warp owns 32 * kItems of them, 32 at a
+// time (ballots rank them, and every load and store is coalesced).  To know how
+// many marked tokens come before its own, a cluster's CTAs split the tokens of
+// all earlier clusters among themselves, add their own counts, and exchange
+// both through distributed shared memory, so nothing waits on another cluster.
+// Bound by latency (launch, one load, one cluster barrier, one store); with
+// kAcMaxClusters clusters each group id is read again six times on average, from
+// L2.  12 clusters are resident at once; with 16 a second wave of clusters cost
+// 20-30 %.  One cluster for the whole layer, as before, left 144 SMs idle.  GPU
+// time of an active set in a row of calls: 6144 tokens 2.9 -> 2.8 us, 75600
+// 6.3 -> 4.0, 524288 26 -> 8.3, 2097152 95 -> 20 (4194304, which took blocks
+// that each counted everything before them, 245 -> 35).
+constexpr int kAcThreads = 1024;
+constexpr int kAcCtas = 8;                             // CTAs of a cluster
+constexpr int kAcMaxClusters = 12;
 
-constexpr int kActThreads = 1024;
-
-template <bool kVec>
-__global__ void __launch_bounds__(kActThreads)
-active_set_kernel(const int32_t *__restrict__ group_of, int N, int K, uint32_t mask, int chunk,
-              int32_t *__restrict__ idx, int32_t *__restrict__ pos, unsigned *err) {
-  __shared__ int warp_cnt[32];
-  __shared__ int block_base;
+// Scans this CTA's rounds: emit(n, g, marked, rank) for every token n < N with
+// its group id g, whether mark(g), and the number of marked tokens before n.
+template <int kItems, class Mark, class Emit>
+__device__ __forceinline__ void compact(const int32_t *__restrict__ group_of, int N, int rounds,
+                                        Mark mark, Emit emit) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ int warp_cnt[2][kAcThreads / 32], warp_before[kAcThreads / 32];
+  __shared__ int own[kAcCtas], earlier[kAcCtas];       // by CTA of the cluster
+  const int cta = (int)cl.block_rank(), ctas = (int)cl.num_blocks();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int start = blockIdx.x * chunk;
-  const int end = min(N, start + chunk);
-  auto act = [&](int g) -> int {
-    return (g >= 0 && g < K) ? (int)((mask >> g) & 1u) : 0;
-  };
-  // 1. active tokens before this chunk
-  int c = 0;
-  if (kVec) {
-    const int4 *g4 = reinterpret_cast<const int4 *>(group_of);
-    for (int i = threadIdx.x; i < start / 4; i += kActThreads) {
-      const int4 v = __ldg(g4 + i);
-      c += act(v.x) + act(v.y) + act(v.z) + act(v.w);
-    }
-  } else {
-    for (int i = threadIdx.x; i < start; i += kActThreads) c += act(__ldg(group_of + i));
-  }
+  const unsigned below = (1u << lane) - 1u;
+  constexpr int kTile = kAcThreads * kItems;
+  const long long per_cta = (long long)rounds * kTile;
+  const long long own0 = (long long)blockIdx.x * per_cta + (w * kItems * 32 + lane);
+  // group ids of this lane's tokens of a round, and the marks of its warp's
+  int g[kItems];
+  unsigned bal[kItems];
+  auto load = [&](int r) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) warp_cnt[w] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int i = 0; i < kActThreads / 32; ++i) s += warp_cnt[i];
-    block_base = s;
-  }
-  __syncthreads();
-  int base = block_base;
-  // 2. compact this chunk, 1024 tokens at a time
-  for (int b0 = start; b0 < end; b0 += kActThreads) {
-    const int n = b0 + threadIdx.x;
-    int flag = 0;
-    if (n < end) {
-      const int g = group_of[n];
-      if (g < 0 || g >= K) set_error(err, kErrIndex);
-      flag = act(g);
+    for (int e = 0; e < kItems; ++e) {
+      const long long n = own0 + (long long)r * kTile + e * 32;
+      g[e] = n < N ? __ldg(group_of + n) : 0;
     }
-    const unsigned bal = __ballot_sync(0xffffffffu, flag);
-    __syncthreads();                                   // warp_cnt reuse
-    if (lane == 0) warp_cnt[w] = __popc(bal);
+    int c = 0;
+#pragma unroll
+    for (int e = 0; e < kItems; ++e) {
+      bal[e] = __ballot_sync(0xffffffffu, own0 + (long long)r * kTile + e * 32 < N && mark(g[e]));
+      c += __popc(bal[e]);
+    }
+    return c;                                          // the same in every lane
+  };
+  int base = 0;                                        // marked tokens before this CTA's
+  int c0 = load(0);
+  if (gridDim.x > 1) {
+    cl.barrier_arrive();                               // this CTA has started
+    int c = c0;
+    for (int r = 1; r < rounds; ++r) c += load(r);
+    if (rounds > 1) c0 = load(0);
+    // the earlier clusters own whole CTAs' worth of tokens, all inside N
+    const long long n_before = (long long)(blockIdx.x / ctas) * per_cta;   // tokens per CTA
+    const int32_t *from = group_of + cta * n_before;
+    int e = 0;
+    if ((reinterpret_cast<uintptr_t>(group_of) & 15) == 0) {   // per_cta is a multiple of 4
+      const int4 *f4 = reinterpret_cast<const int4 *>(from);
+#pragma unroll 8
+      for (long long i = threadIdx.x; i < n_before / 4; i += kAcThreads) {
+        const int4 v = __ldg(f4 + i);
+        e += (int)mark(v.x) + (int)mark(v.y) + (int)mark(v.z) + (int)mark(v.w);
+      }
+    } else {
+#pragma unroll 8
+      for (long long i = threadIdx.x; i < n_before; i += kAcThreads) e += (int)mark(__ldg(from + i));
+    }
+    e = __reduce_add_sync(0xffffffffu, e);
+    if (lane == 0) {
+      warp_cnt[0][w] = c;
+      warp_before[w] = e;
+    }
+    cl.barrier_wait();                                 // every CTA has, so its memory exists
     __syncthreads();
-    int before = 0, total = 0;
-    for (int i = 0; i < kActThreads / 32; ++i) {
-      const int v = warp_cnt[i];
-      before += (i < w) ? v : 0;
-      total += v;
+    if (w == 0) {
+      c = __reduce_add_sync(0xffffffffu, warp_cnt[0][lane]);
+      e = __reduce_add_sync(0xffffffffu, warp_before[lane]);
+      if (lane < ctas) {
+        *cl.map_shared_rank(&own[cta], lane) = c;
+        *cl.map_shared_rank(&earlier[cta], lane) = e;
+      }
     }
-    const int r = base + before + __popc(bal & ((1u << lane) - 1u));
-    if (n < end) {
-      if (flag) idx[r] = n;
-      if (pos) pos[n] = flag ? r : -1;
+    cl.sync();                                         // every CTA's counts have arrived
+    for (int r = 0; r < ctas; ++r) base += earlier[r] + (r < cta ? own[r] : 0);
+  }
+  for (int r = 0; r < rounds; ++r) {
+    if (r > 0) c0 = load(r);
+    // two buffers: a warp writes the next round's count only after every warp
+    // has passed this round's barrier
+    if (lane == 0) warp_cnt[(r + 1) & 1][w] = c0;
+    __syncthreads();
+    const int wc = warp_cnt[(r + 1) & 1][lane];
+    int rank = base + __reduce_add_sync(0xffffffffu, lane < w ? wc : 0);
+    base += __reduce_add_sync(0xffffffffu, wc);
+#pragma unroll
+    for (int e = 0; e < kItems; ++e) {
+      const long long n = own0 + (long long)r * kTile + e * 32;
+      if (n < N) emit((int)n, g[e], bal[e] >> lane & 1u, rank + __popc(bal[e] & below));
+      rank += __popc(bal[e]);
     }
-    base += total;
   }
 }
 
-// Active set of layers up to kAcMaxN tokens in one cluster of kCsCtas CTAs:
-// CTA c owns tokens [c*chunk, (c+1)*chunk).  First pass: each CTA marks its
-// active tokens (one bit each, in shared memory) and counts them.  The CTAs
-// exchange their counts through distributed shared memory (CTA order is token
-// order), so CTA c learns how many active tokens come before its range; the
-// second pass compacts from the bits.  Group ids are read once, and no global
-// scratch or inter-CTA spin is needed.
-constexpr int kAcThreads = 1024;
-constexpr int kAcMaxChunk = 256 * 1024;                // tokens per CTA: 32 KB of bits
-constexpr int kAcMaxN = kCsCtas * kAcMaxChunk;         // 2097152 tokens
-
-__global__ void __cluster_dims__(kCsCtas, 1, 1) __launch_bounds__(kAcThreads, 1)
-active_set_cluster_kernel(const int32_t *__restrict__ group_of, int N, int K, uint32_t mask,
-                          int chunk, int32_t *__restrict__ idx, int32_t *__restrict__ pos,
-                          unsigned *err) {
+template <int kItems>
+__global__ void __launch_bounds__(kAcThreads, 1)
+active_set_kernel(const int32_t *__restrict__ group_of, int N, int rounds, int K, uint32_t mask,
+                  int32_t *__restrict__ idx, int32_t *__restrict__ pos, unsigned *err) {
   pdl_wait();
   pdl_trigger();
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  __shared__ uint32_t bits[kAcMaxChunk / 32];          // bit t: token lo + t is active
-  __shared__ int warp_cnt[kAcThreads / 32];
-  __shared__ int cta_count;
-  __shared__ int cta_base;
-  const int cta = (int)cl.block_rank();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int lo = min(N, cta * chunk), hi = min(N, lo + chunk);
-  const int n_loc = hi - lo;
-  const int rounds = (n_loc + kAcThreads - 1) / kAcThreads;
-  auto act = [&](int g) -> int { return (g >= 0 && g < K) ? (int)((mask >> g) & 1u) : 0; };
-  // pass 1: bits and count; four rounds' loads are issued before their ballots
-  int c = 0;
-  for (int r0 = 0; r0 < rounds; r0 += 4) {
-    int g[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int t = (r0 + u) * kAcThreads + threadIdx.x;
-      g[u] = t < n_loc ? __ldg(group_of + lo + t) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (r0 + u >= rounds) break;                     // uniform across the block
-      const int t = (r0 + u) * kAcThreads + threadIdx.x;
-      int flag = 0;
-      if (t < n_loc) {
-        if (g[u] < 0 || g[u] >= K) set_error(err, kErrIndex);
-        flag = act(g[u]);
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, flag);
-      if (lane == 0) {
-        bits[(r0 + u) * (kAcThreads / 32) + w] = bal;
-        c += __popc(bal);
-      }
-    }
-  }
-  if (lane == 0) warp_cnt[w] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int i = 0; i < kAcThreads / 32; ++i) s += warp_cnt[i];
-    cta_count = s;
-  }
-  cl.sync();                                           // every CTA's count is known
-  if (threadIdx.x == 0) {
-    int b = 0;
-    for (int r = 0; r < cta; ++r) b += *cl.map_shared_rank(&cta_count, r);
-    cta_base = b;
-  }
-  cl.sync();                  // no CTA exits while another still reads its count
-  // pass 2: compact from the bits, one round of kAcThreads tokens at a time
-  int base = cta_base;
-  for (int r = 0; r < rounds; ++r) {
-    const int t = r * kAcThreads + threadIdx.x;
-    const unsigned bal = bits[r * (kAcThreads / 32) + w];
-    // active tokens of the round's earlier warps: lane i holds warp i's count,
-    // an inclusive warp scan gives every prefix
-    const int cnt = __popc(bits[r * (kAcThreads / 32) + lane]);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const int before = __shfl_sync(0xffffffffu, incl - cnt, w);
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    const int flag = (bal >> lane) & 1u;
-    const int rank = base + before + __popc(bal & ((1u << lane) - 1u));
-    if (t < n_loc) {
-      if (flag) idx[rank] = lo + t;
-      if (pos) pos[lo + t] = flag ? rank : -1;
-    }
-    base += total;
-  }
+  compact<kItems>(
+      group_of, N, rounds,
+      [&](int g) { return (unsigned)g < (unsigned)K && (mask >> g & 1u); },
+      [&](int n, int g, bool active, int rank) {
+        if ((unsigned)g >= (unsigned)K) set_error(err, kErrIndex);
+        if (active) idx[rank] = n;
+        if (pos) pos[n] = active ? rank : -1;
+      });
+}
+
+template <int kItems>
+__global__ void __launch_bounds__(kAcThreads, 1)
+reorder_kernel(const int32_t *__restrict__ group_of, int N, int rounds, int M,
+               int32_t *__restrict__ order, int32_t *__restrict__ where,
+               int32_t *__restrict__ group_new, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
+  compact<kItems>(
+      group_of, N, rounds, [&](int g) { return g != 0; },
+      [&](int n, int g, bool moved, int rank) {
+        // n - rank baseline tokens come before n
+        const long long r = moved ? rank : (long long)M + (n - rank);
+        if (moved ? rank < M : r < N) {
+          order[r] = n;
+          if (where) where[n] = (int)r;
+          if (group_new) group_new[r] = g;
+        } else {
+          set_error(err, kErrIndex);
+        }
+      });
 }
 
 }  // namespace
@@ -835,11 +822,31 @@ bool cluster_ready(int ctas, int threads) {
   return st == 1;
 }
 
-bool cluster_active_ready() {
-  return cluster_ready<active_set_cluster_kernel>(kCsCtas, kAcThreads);
-}
-
 bool cluster_scan_ready() { return cluster_ready<radix_scan_kernel>(kScanCtas, 1024); }
+
+// Launches a compaction kernel over N tokens: one CTA where one round of it
+// covers them (1.3 us against 2.6 for a cluster), else clusters; one token per
+// thread and round while a single cluster covers the layer that way (8192
+// tokens; 6144: 2.8 us against 3.4 with four), four otherwise (fewer barriers
+// per token); one round per CTA until kAcMaxClusters are in flight, then more.  Without
+// room for a cluster of 8, clusters of one CTA.
+template <auto Kernel1, auto Kernel4, typename... Rest>
+void launch_compact(cudaStream_t s, const int32_t *group_of, int N, Rest... rest) {
+  const bool one = N <= kAcCtas * kAcThreads;
+  const long long tile = one ? kAcThreads : 4 * kAcThreads;
+  const long long tiles = ((long long)N + tile - 1) / tile;
+  unsigned ctas = 1;
+  long long rounds = 1, grid = 1;
+  if (tiles > 1) {
+    ctas = cluster_ready<Kernel4>(kAcCtas, kAcThreads) ? kAcCtas : 1;
+    const long long most = (long long)kAcMaxClusters * kAcCtas;
+    rounds = (tiles + most - 1) / most;
+    grid = (tiles + rounds * ctas - 1) / (rounds * ctas) * ctas;
+  }
+  count_launches(1);
+  launch_pdl_cluster(one ? Kernel1 : Kernel4, dim3((unsigned)grid), dim3(kAcThreads), ctas, s,
+                     group_of, N, (int)rounds, rest...);
+}
 
 }  // namespace
 
@@ -932,101 +939,10 @@ extern "C" int hsa_partition_active(const int32_t *group_of, int N, int T, const
     const bool full = iter < m || iter > T - m - 1;
     if (full || iter % (T / budgets[k]) == 0) mask |= 1u << k;
   }
-  cudaStream_t s = (cudaStream_t)stream;
   unsigned *err = device_error_word();
   if (!err) return HSA_ERR_CUDA;
-  if (N <= kAcMaxN && cluster_active_ready()) {
-    const int chunk = (N + kCsCtas - 1) / kCsCtas;
-    count_launches(1);
-    launch_pdl(active_set_cluster_kernel, dim3(kCsCtas), dim3(kAcThreads), 0, s, group_of, N, K,
-               mask, chunk, idx, pos, err);
-    return launch_status();
-  }
-  // Larger layers: chunks of whole 1024-token rounds, at most one block per
-  // SM; block b counts the active tokens of the chunks before its own.
-  const int sms = sm_count();
-  long long chunk = ((long long)N + sms - 1) / sms;
-  chunk = ((chunk + kActThreads - 1) / kActThreads) * kActThreads;
-  const int blocks = (int)(((long long)N + chunk - 1) / chunk);
-  count_launches(1);
-  if (aligned16(group_of))
-    active_set_kernel<true><<<blocks, kActThreads, 0, s>>>(group_of, N, K, mask, (int)chunk, idx,
-                                                        pos, err);
-  else
-    active_set_kernel<false><<<blocks, kActThreads, 0, s>>>(group_of, N, K, mask, (int)chunk, idx,
-                                                         pos, err);
+  launch_compact<active_set_kernel<1>, active_set_kernel<4>>((cudaStream_t)stream, group_of, N, K, mask, idx, pos, err);
   return launch_status();
-}
-
-// ------------------------------------------------------- token reordering
-//
-// Sec. 2.5: new position r holds old token order[r]; non-baseline tokens
-// (group != 0) first, then the baseline group, each in token order.  Same
-// workspace-free scheme as the active set: block b counts the non-baseline
-// tokens before its chunk, then ranks its chunk with warp ballots.
-
-template <bool kVec>
-__global__ void __launch_bounds__(kActThreads)
-reorder_kernel(const int32_t *__restrict__ group_of, int N, int M, int chunk,
-               int32_t *__restrict__ order, int32_t *__restrict__ where,
-               int32_t *__restrict__ group_new, unsigned *err) {
-  __shared__ int warp_cnt[32];
-  __shared__ int block_base;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int start = blockIdx.x * chunk;
-  const int end = min(N, start + chunk);
-  int c = 0;
-  if (kVec) {
-    const int4 *g4 = reinterpret_cast<const int4 *>(group_of);
-    for (int i = threadIdx.x; i < start / 4; i += kActThreads) {
-      const int4 v = __ldg(g4 + i);
-      c += (v.x != 0) + (v.y != 0) + (v.z != 0) + (v.w != 0);
-    }
-  } else {
-    for (int i = threadIdx.x; i < start; i += kActThreads) c += __ldg(group_of + i) != 0;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) warp_cnt[w] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int i = 0; i < kActThreads / 32; ++i) s += warp_cnt[i];
-    block_base = s;
-  }
-  __syncthreads();
-  int nb_base = block_base;             // non-baseline tokens before b0
-  for (int b0 = start; b0 < end; b0 += kActThreads) {
-    const int n = b0 + threadIdx.x;
-    int g = 0, flag = 0;
-    if (n < end) {
-      g = group_of[n];
-      flag = g != 0;
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, flag);
-    __syncthreads();
-    if (lane == 0) warp_cnt[w] = __popc(bal);
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int i = 0; i < kActThreads / 32; ++i) {
-      const int v = warp_cnt[i];
-      before += (i < w) ? v : 0;
-      total += v;
-    }
-    if (n < end) {
-      const int nb_rank = nb_base + before + __popc(bal & ((1u << lane) - 1u));
-      // baseline rank = tokens before n that are baseline
-      const int r = flag ? nb_rank : M + (n - nb_rank);
-      if ((flag && nb_rank < M) || (!flag && r < N)) {
-        order[r] = n;
-        if (where) where[n] = r;
-        if (group_new) group_new[r] = g;
-      } else {
-        set_error(err, kErrIndex);
-      }
-    }
-    nb_base += total;
-  }
 }
 
 // ------------------------------------------------- allocation strategies
@@ -1129,19 +1045,7 @@ extern "C" int hsa_reorder_tokens(const int32_t *group_of, int N, int n_baseline
   if (!group_of || !order) return HSA_ERR_INVALID_ARG;
   unsigned *err = device_error_word();
   if (!err) return HSA_ERR_CUDA;
-  const int sms = sm_count();
-  long long chunk = ((long long)N + sms - 1) / sms;
-  chunk = ((chunk + kActThreads - 1) / kActThreads) * kActThreads;
-  if (chunk < 4096) chunk = 4096;
-  const int blocks = (int)(((long long)N + chunk - 1) / chunk);
-  const int M = N - n_baseline;
-  cudaStream_t s = (cudaStream_t)stream;
-  count_launches(1);
-  if (aligned16(group_of))
-    reorder_kernel<true><<<blocks, kActThreads, 0, s>>>(group_of, N, M, (int)chunk, order, where,
-                                                         group_new, err);
-  else
-    reorder_kernel<false><<<blocks, kActThreads, 0, s>>>(group_of, N, M, (int)chunk, order, where,
-                                                          group_new, err);
+  launch_compact<reorder_kernel<1>, reorder_kernel<4>>((cudaStream_t)stream, group_of, N, N - n_baseline, order, where,
+                                 group_new, err);
   return launch_status();
 }
