@@ -6,10 +6,10 @@
 // unsigned key whose integer order is the float order (-0 folded onto +0); the
 // rank of a token is its position in the (key, token) order, which is the tie
 // rule, and rank r maps to its group.  Three paths give the same groups:
-//   N <= 12032    one launch ranks every token by counting the pairs before it;
+//   N <= 4864     one launch ranks every token by counting the pairs before it;
 //   N <= 360448   one launch of a cluster of 8 CTAs (keys spread over their
-//                 shared memory) finds the pair at each group boundary by radix
-//                 select and compares every token with those pairs;
+//                 shared memory) finds the pair at each group boundary and
+//                 compares every token with those pairs;
 //   larger N      a least-significant-digit radix sort of the (key, token)
 //                 pairs: four passes of 8 bits, each a per-tile histogram, one
 //                 exclusive scan of the (digit, tile) counts in digit-major
@@ -272,13 +272,15 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
 // (ties count) before them and kn (ties do not) behind them: two instructions
 // per key and a quarter of a 16-byte broadcast load, instead of the five of
 // the general pair test on single words.  Calls in a row (GPU time of a graph
-// of 20): N = 6144 22.4 -> 8.9 us, N = 12032 60 -> 28 us.
+// of 20): N = 3000 8.2 -> 3.8 us.
 constexpr int kRankThreads = 512;
 constexpr int kRankWarps = kRankThreads / 32;
 constexpr int kRankTokens = 32;
 // The keys (dynamic, whole 16-byte vectors) and the partial counts (static)
 // stay within the 48 KB a block gets without opting in to more shared memory.
-constexpr int kRankMaxN = 12032;
+// One block per SM is the limit: 4500 tokens 4.9 us against 7.5 for the select
+// below, 6144 tokens (a second block on some SMs) 8.9 against 8.0.
+constexpr int kRankMaxN = 152 * kRankTokens;           // 4864
 static_assert(kRankMaxN % 4 == 0 && kRankMaxN * 4 + kRankTokens * 4 <= 48 * 1024,
               "rank partition shared memory");
 
@@ -355,55 +357,81 @@ rank_partition_kernel(const float *__restrict__ stat, int N, int K, GroupStarts 
 // rank >= start[k] for k = 0 .. K-2 (group K-1 holds the lowest ranks), and
 // rank >= b holds exactly when (key, token) >= the pair of rank b in the
 // (key, token) order.  So it is enough to find the pair of each boundary rank
-// (a radix select: four 8-bit digit passes, each a histogram of the keys that
-// share the boundary's digits so far, then the boundary's position among the
-// keys equal to its key, counted in token order) and to compare every token
-// with those pairs: one launch instead of a sort's fourteen, and the same
-// ranks as the stable sort.
+// and to compare every token with those pairs: one launch instead of a sort's
+// fourteen, and the same ranks as the stable sort.
+//
+// It runs on one thread-block cluster.  CTA c holds the keys of tokens
+// [c*chunk, (c+1)*chunk) in its shared memory.
+//   1. The cluster's smallest and largest key.
+//   2. A histogram of 2048 or 4096 bins over that range (2^s keys each); every
+//      CTA sums the cluster's through distributed shared memory and finds each
+//      boundary's bin (identical integer work on identical data, so no broadcast
+//      is needed).  The bins follow the values at hand, so they hold few keys
+//      (a lognormal statistic of 75600 tokens: about 120 at a quartile) and
+//      their counters seldom collide.
+//   3. The keys of a boundary's bin, with their tokens, go to the list of the
+//      CTA that owns the boundary (boundary j: CTA j mod 8), which finds the
+//      pair with the right number of smaller pairs and writes it to every CTA.
+// A bin with more than kCsList keys is split further first, 256 ways per pass,
+// until it holds fewer or a single key value; a value that more tokens share is
+// resolved by counting it in token order (CTA order is token order).
+// Cluster barriers are hardware barriers that every thread of every CTA
+// reaches, so none can wait forever.  Latency-bound (8 SMs, four cluster
+// barriers): 12033 tokens 26.8 -> 8.3 us, 75600 43 -> 13.8, 360448
+// 110 -> 37, against four fixed 8-bit digit passes with two barriers each and bins
+// that most keys shared.  Of the 75600 tokens' 12 us in the kernel, reading the
+// eight histograms takes 2, the two sweeps and the lists 5.
 constexpr int kMaxBounds = kMaxGroups - 1;
-
-// The select runs on a thread-block cluster of
-// kCsCtas CTAs (one launch).  CTA c holds the keys of tokens [c*chunk,
-// (c+1)*chunk) in its shared memory; each digit pass builds one histogram per
-// CTA, and every CTA then sums the cluster's histograms through distributed
-// shared memory and takes the same digit decisions (identical integer work on
-// identical data, so no broadcast is needed).  The boundary token is found in
-// the CTA whose token range holds it (counts of equal keys are exchanged the
-// same way, in CTA order = token order); that CTA writes the boundary pair into
-// every CTA's shared memory.  Cluster barriers are hardware barriers: every
-// thread of every CTA reaches each of them, so none can wait forever.
 constexpr int kCsCtas = 8;
 constexpr int kCsThreads = 1024;
 constexpr int kCsMaxChunk = 44 * 1024;                 // keys per CTA: 176 KB
 constexpr int kCsMaxN = kCsCtas * kCsMaxChunk;         // 360448 tokens
+constexpr int kCsFineN = 98304;                        // above: 4096 bins
+constexpr int kCsList = 512;                           // pairs a boundary's list holds
+constexpr int kCsLists = (kMaxBounds + kCsCtas - 1) / kCsCtas;   // boundaries a CTA owns
+constexpr int kCsHist = kMaxBounds * 256;              // counters, 4096 in the first histogram
+static_assert(kCsList * 2 == kCsThreads && kCsHist >= 4 * kCsThreads, "select layout");
+constexpr int kCsFixedBytes = kCsHist * 4 + kCsLists * kCsList * 8;   // besides the keys
 
+// kPer: bins per thread of the first histogram.
+template <int kPer>
 __global__ void __cluster_dims__(kCsCtas, 1, 1) __launch_bounds__(kCsThreads, 1)
 cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, GroupStarts gs,
                       int32_t *__restrict__ group_of, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ uint4 ckey4[];                     // this CTA's keys, padded to uint4
+  extern __shared__ uint4 cs_smem[];
+  unsigned long long *list = reinterpret_cast<unsigned long long *>(cs_smem);
+  uint32_t *hist = reinterpret_cast<uint32_t *>(list + kCsLists * kCsList);
+  uint4 *ckey4 = reinterpret_cast<uint4 *>(hist + kCsHist);   // this CTA's keys
   uint32_t *skey = reinterpret_cast<uint32_t *>(ckey4);
-  __shared__ __align__(16) uint32_t hist[kMaxBounds * 256];   // [prefix slot][digit]
-  __shared__ uint32_t pre[kMaxBounds];                 // boundary key digits found so far
-  __shared__ int below[kMaxBounds];                    // keys ordered below that prefix
-  __shared__ int slot[kMaxBounds];                     // histogram of the boundary's prefix
-  __shared__ uint32_t dpre[kMaxBounds];                // distinct prefixes, ascending
-  __shared__ int nd;
-  __shared__ int eqc[kMaxBounds];                      // local keys equal to a boundary key
+  __shared__ uint2 range[kCsCtas];                     // every CTA's smallest, largest key
+  __shared__ uint32_t low[kMaxBounds];                 // boundary j's keys: [low, low + 2^sh)
+  __shared__ int sh[kMaxBounds];
+  __shared__ int below[kMaxBounds];                    // keys below low
+  __shared__ int count[kMaxBounds];                    // keys in the range
+  __shared__ int fill[kMaxBounds];                     // place of this CTA's next pair of them
+  __shared__ int slot[kMaxBounds];                     // first boundary with the same range
+  __shared__ int target[kMaxBounds];                   // boundary's rank; -1: 0 or N
+  __shared__ int split;                                // whether a range holds too many keys
   __shared__ unsigned long long thr[kMaxBounds];       // boundary pair (key << 32 | token)
+  __shared__ int eqc[kMaxBounds];                      // local keys equal to a boundary key
   __shared__ int warp_tot[kCsThreads / 32];
+  __shared__ uint32_t warp_min[kCsThreads / 32], warp_max[kCsThreads / 32];
+  cl.barrier_arrive();                                 // this CTA has started
   const int cta = (int)cl.block_rank();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nb = K - 1;
   const int lo = min(N, cta * chunk), hi = min(N, lo + chunk);
   const int n_loc = hi - lo;
   const int n4 = (n_loc + 3) >> 2;
-  auto searched = [&](int j) { return gs.start[j] > 0 && gs.start[j] < N; };
-
   // keys of [lo, hi); chunk is a multiple of 4, so a 16-byte aligned stat
   // gives 16-byte aligned rows
   const bool vec = (reinterpret_cast<uintptr_t>(stat) & 15) == 0;
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll 4
   for (int i = threadIdx.x; i < n4; i += kCsThreads) {
     float f[4];
     if (vec && 4 * i + 3 < n_loc) {
@@ -411,145 +439,240 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
       f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) f[e] = 4 * i + e < n_loc ? __ldg(stat + lo + 4 * i + e) : 0.f;
+      for (int e = 0; e < 4; ++e)                      // past the end: the last key again
+        f[e] = __ldg(stat + lo + min(4 * i + e, n_loc - 1));
     }
     if (!(isfinite(f[0]) && isfinite(f[1]) && isfinite(f[2]) && isfinite(f[3])))
       set_error(err, kErrNonfinite);
-    ckey4[i] = make_uint4(order_key(f[0]), order_key(f[1]), order_key(f[2]), order_key(f[3]));
+    const uint4 k = make_uint4(order_key(f[0]), order_key(f[1]), order_key(f[2]), order_key(f[3]));
+    kmin = min(kmin, min(min(k.x, k.y), min(k.z, k.w)));
+    kmax = max(kmax, max(max(k.x, k.y), max(k.z, k.w)));
+    ckey4[i] = k;
   }
-  if (threadIdx.x == 0) {
-    nd = 1;
-    dpre[0] = 0u;
-  }
-  if (threadIdx.x < kMaxBounds) {
-    pre[threadIdx.x] = 0u;
-    below[threadIdx.x] = 0;
-    slot[threadIdx.x] = 0;
-    eqc[threadIdx.x] = 0;
-  }
-  __syncthreads();
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
-    const int n_hist = nd;
-    for (int i = threadIdx.x; i < n_hist * 256; i += kCsThreads) hist[i] = 0u;
-    __syncthreads();
-    // Local histogram.  Every lane of a warp runs the same number of rounds,
-    // so the warp can merge equal bins (__match_any_sync) and add each bin's
-    // count once: in early passes most keys share a few bins.
-    for (int b4 = 0; b4 < n4; b4 += kCsThreads) {
-      const int i = b4 + threadIdx.x;
-      uint4 k4 = make_uint4(0u, 0u, 0u, 0u);
-      if (i < n4) k4 = ckey4[i];
-      const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t bin = 0xffffffffu;                    // no histogram
-        if (i < n4 && 4 * i + e < n_loc) {
-          const uint32_t key = kk[e];
-          const uint32_t hp = pass == 0 ? 0u : key >> (shift + 8);
-          for (int q = 0; q < n_hist; ++q) {           // few distinct prefixes
-            const uint32_t v = dpre[q];
-            if (v >= hp) {
-              if (v == hp) bin = (uint32_t)q * 256u + ((key >> shift) & 255u);
-              break;
-            }
-          }
+  for (int i = 0; i < kPer; ++i) hist[i * kCsThreads + threadIdx.x] = 0u;
+  if (threadIdx.x < nb) {
+    const int r = gs.start[threadIdx.x];
+    target[threadIdx.x] = r > 0 && r < N ? r : -1;
+    thr[threadIdx.x] = r <= 0 ? 0ull : ~0ull;
+    eqc[threadIdx.x] = 0;
+    count[threadIdx.x] = 0;
+    fill[threadIdx.x] = kCsList;
+  }
+  if (threadIdx.x == 0) split = 0;
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) {
+    warp_min[w] = kmin;
+    warp_max[w] = kmax;
+  }
+  cl.barrier_wait();                                   // every CTA has, so its memory exists
+  __syncthreads();
+  if (w == 0) {
+    kmin = __reduce_min_sync(0xffffffffu, warp_min[lane]);
+    kmax = __reduce_max_sync(0xffffffffu, warp_max[lane]);
+    if (lane < kCsCtas) *cl.map_shared_rank(&range[cta], lane) = make_uint2(kmin, kmax);
+  }
+  cl.sync();                                           // every CTA's range has arrived
+#pragma unroll
+  for (int r = 0; r < kCsCtas; ++r) {
+    kmin = r ? min(kmin, range[r].x) : range[0].x;
+    kmax = r ? max(kmax, range[r].y) : range[0].y;
+  }
+  // bins of 2^s keys: (kmax - kmin) >> s < 1024 * kPer
+  int s = max(0, (kPer == 4 ? 20 : 21) - __clz(kmax - kmin));
+  for (int i = threadIdx.x; i < n4; i += kCsThreads) {
+    const uint4 k4 = ckey4[i];
+    const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (4 * i + e < n_loc) atomicAdd(&hist[(kk[e] - kmin) >> s], 1u);
+  }
+  cl.sync();                                           // every CTA's histogram is complete
+  {
+    // thread t: bins kPer*t .. of the cluster's histogram, then their prefix
+    uint32_t hv[kCsCtas][kPer];
+#pragma unroll
+    for (int r = 0; r < kCsCtas; ++r) {
+      const uint32_t *h = cl.map_shared_rank(hist, r) + kPer * threadIdx.x;
+      if constexpr (kPer == 4)
+        *reinterpret_cast<uint4 *>(hv[r]) = *reinterpret_cast<const uint4 *>(h);
+      else
+        *reinterpret_cast<uint2 *>(hv[r]) = *reinterpret_cast<const uint2 *>(h);
+    }
+    int c[kPer], before[kPer], sum = 0;                // before: in earlier CTAs
+#pragma unroll
+    for (int b = 0; b < kPer; ++b) {
+      c[b] = before[b] = 0;
+#pragma unroll
+      for (int r = 0; r < kCsCtas; ++r) {
+        c[b] += (int)hv[r][b];
+        before[b] += r < cta ? (int)hv[r][b] : 0;
+      }
+      sum += c[b];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) warp_tot[w] = incl;
+    __syncthreads();
+    const int wt = warp_tot[lane];
+    const int excl = __reduce_add_sync(0xffffffffu, lane < w ? wt : 0) + incl - sum;
+    for (int j = 0; j < nb; ++j) {
+      int t = target[j] - excl;                        // ranks 0 and N fall in no bin
+      if (t < 0 || t >= sum) continue;
+#pragma unroll
+      for (int b = 0; b < kPer; ++b) {
+        if (t >= 0 && t < c[b]) {
+          low[j] = kmin + ((uint32_t)(kPer * threadIdx.x + b) << s);
+          sh[j] = s;
+          below[j] = target[j] - t;
+          count[j] = c[b];
+          fill[j] = before[b];
+          if (c[b] > kCsList && s > 0) split = 1;
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        if (bin != 0xffffffffu && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+        t -= c[b];
       }
     }
-    cl.sync();                                         // every CTA's histogram is complete
-    // warp j picks boundary j's digit from the cluster's summed histogram
-    if (w < nb && searched(w)) {
-      const int target = gs.start[w] - below[w];       // rank among the prefix's keys
-      // bins 8*lane .. 8*lane+7 of every CTA's histogram: all 16 remote
-      // 16-byte loads are issued before they are summed
-      uint4 hv[kCsCtas][2];
+  }
+  __syncthreads();
+  // Split the ranges that hold too many keys, 256 ways at a time.  All of them
+  // are 2^s wide here, and every thread of the cluster takes the same turns.
+  while (__builtin_expect(split, 0)) {
+    const int ns = max(0, s - 8);
+    if (threadIdx.x < nb) {
+      const int j = threadIdx.x;
+      int first = -1;
+      if (target[j] >= 0 && count[j] > kCsList && sh[j] == s) {
+        first = 0;
+        while (!(target[first] >= 0 && sh[first] == s && low[first] == low[j])) ++first;
+      }
+      slot[j] = first;                                 // -1: not split
+    }
+    cl.sync();                  // every CTA has read the histograms of the last pass
+    if (threadIdx.x == 0) split = 0;
+    for (int i = threadIdx.x; i < nb * 256; i += kCsThreads) hist[i] = 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_loc; i += kCsThreads) {
+      const uint32_t k = skey[i];
+      for (int j = 0; j < nb; ++j)
+        if (slot[j] == j && (k - low[j]) >> s == 0)
+          atomicAdd(&hist[j * 256 + ((k - low[j]) >> ns)], 1u);
+    }
+    cl.sync();                                         // every CTA's histograms are complete
+    // warp j picks boundary j's part of its range
+    if (w < nb && slot[w] >= 0) {
+      const int t = target[w] - below[w];              // rank among the range's keys
+      int c[8], before[8], sum = 0;
 #pragma unroll
+      for (int i = 0; i < 8; ++i) c[i] = before[i] = 0;
       for (int r = 0; r < kCsCtas; ++r) {
         const uint4 *h = reinterpret_cast<const uint4 *>(cl.map_shared_rank(hist, r) +
                                                          slot[w] * 256 + 8 * lane);
-        hv[r][0] = h[0];
-        hv[r][1] = h[1];
-      }
-      int c[8], sum = 0;
+        const uint4 h0 = h[0], h1 = h[1];
+        const int v[8] = {(int)h0.x, (int)h0.y, (int)h0.z, (int)h0.w,
+                          (int)h1.x, (int)h1.y, (int)h1.z, (int)h1.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) c[i] = 0;
-#pragma unroll
-      for (int r = 0; r < kCsCtas; ++r) {
-        c[0] += (int)hv[r][0].x; c[1] += (int)hv[r][0].y; c[2] += (int)hv[r][0].z;
-        c[3] += (int)hv[r][0].w; c[4] += (int)hv[r][1].x; c[5] += (int)hv[r][1].y;
-        c[6] += (int)hv[r][1].z; c[7] += (int)hv[r][1].w;
+        for (int i = 0; i < 8; ++i) {
+          c[i] += v[i];
+          before[i] += r < cta ? v[i] : 0;
+        }
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) sum += c[i];
       int incl = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
       }
-      const int excl = incl - sum;
-      if (target >= excl && target < incl) {           // exactly one lane
-        int cum = excl, d = 8 * lane;
+      __syncwarp();                                    // every lane has read low and below
+      int at = t - (incl - sum);
+      if (at >= 0 && at < sum) {                       // exactly one lane
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (target < cum + c[i]) { d = 8 * lane + i; break; }
-          cum += c[i];
+        for (int d = 0; d < 8; ++d) {
+          if (at >= 0 && at < c[d]) {
+            low[w] += (uint32_t)(8 * lane + d) << ns;
+            sh[w] = ns;
+            below[w] = target[w] - at;
+            count[w] = c[d];
+            fill[w] = before[d];
+            if (c[d] > kCsList && ns > 0) split = 1;
+          }
+          at -= c[d];
         }
-        pre[w] = (pre[w] << 8) | (uint32_t)d;
-        below[w] += cum;                               // keys below the longer prefix
       }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {                            // distinct prefixes, ascending
-      int m = 0;
-      for (int j = 0; j < nb; ++j) {
-        if (!searched(j)) continue;
-        const uint32_t v = pre[j];
-        int p = 0;
-        while (p < m && dpre[p] < v) ++p;
-        if (p == m || dpre[p] != v) {
-          for (int q = m; q > p; --q) dpre[q] = dpre[q - 1];
-          dpre[p] = v;
-          ++m;
+    s = ns;
+  }
+  // The pairs of each boundary's range go to its owner's list, after those of
+  // earlier CTAs (the histograms say how many); a single key value that more
+  // than kCsList tokens share is only counted.
+  // Four boundaries per sweep, held in registers.
+  for (int j0 = 0; j0 < nb; j0 += 4) {
+    uint32_t l[4];
+    int b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const bool on = j0 + q < nb && target[j0 + q] >= 0;
+      l[q] = on ? low[j0 + q] : 0xffffffffu;           // no finite value's key
+      b[q] = on ? sh[j0 + q] : 0;
+    }
+    for (int i = threadIdx.x; i < n4; i += kCsThreads) {
+      const uint4 k4 = ckey4[i];
+      const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if ((kk[e] - l[q]) >> b[q] != 0 || 4 * i + e >= n_loc || j0 + q >= nb) continue;
+          const int j = j0 + q;
+          if (count[j] > kCsList) {
+            atomicAdd(&eqc[j], 1);
+          } else {
+            const int at = atomicAdd(&fill[j], 1);
+            if (at < kCsList)            // more only with a NaN among the keys
+              *cl.map_shared_rank(&list[(j / kCsCtas) * kCsList + at], j % kCsCtas) =
+                  ((unsigned long long)kk[e] << 32) | (unsigned)(lo + 4 * i + e);
+          }
         }
       }
-      for (int j = 0; j < nb; ++j) {
-        if (!searched(j)) continue;
-        int p = 0;
-        while (dpre[p] != pre[j]) ++p;
-        slot[j] = p;
-      }
-      nd = m > 0 ? m : 1;
     }
-    cl.sync();                // no CTA clears its histogram while another reads it
   }
-  // Keys equal to each boundary key in this CTA: one sweep over a contiguous
-  // run of tokens per thread (an odd run length spreads a warp's reads over
-  // the shared-memory banks).
+  cl.sync();                                           // the lists and eqc are complete
+  bool shared_value = false;
+  for (int j = 0; j < nb; ++j) shared_value |= target[j] >= 0 && count[j] > kCsList;
+  for (int j = cta; j < nb; j += kCsCtas) {
+    if (target[j] < 0 || count[j] > kCsList) continue;
+    // 2^lg neighbouring threads per candidate, each a part of the list
+    const unsigned long long *l = list + (j / kCsCtas) * kCsList;
+    const int m = count[j], need = target[j] - below[j];
+    const int lg = min(5, __clz(max(m - 1, 1)) - 22);  // m <= 2^(10 - lg)
+    const int c = threadIdx.x >> lg, part = threadIdx.x & ((1 << lg) - 1);
+    const unsigned long long pair = l[min(c, m - 1)];
+    int less = 0;
+#pragma unroll 8
+    for (int i = part; i < m; i += 1 << lg) less += l[i] < pair;
+    for (int o = 1; o < 1 << lg; o <<= 1) less += __shfl_xor_sync(0xffffffffu, less, o);
+    if (c < m && less == need)
+      for (int r = part; r < kCsCtas; r += 1 << lg) *cl.map_shared_rank(&thr[j], r) = pair;
+  }
+  // A shared value: the need-th of its tokens, in token order.  One sweep over
+  // a contiguous run of tokens per thread (an odd run length spreads a warp's
+  // reads over the shared-memory banks).
   const int run = ((n_loc + kCsThreads - 1) / kCsThreads) | 1;
-  const int r0 = min(n_loc, threadIdx.x * run), r1 = min(n_loc, r0 + run);
-  for (int j = 0; j < nb; ++j) {
-    if (!searched(j)) continue;
-    const uint32_t kj = pre[j];
-    int eq = 0;
-    for (int n = r0; n < r1; ++n) eq += skey[n] == kj;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) eq += __shfl_xor_sync(0xffffffffu, eq, o);
-    if (lane == 0 && eq) atomicAdd(&eqc[j], eq);
-  }
-  for (int j = threadIdx.x; j < nb; j += kCsThreads)
-    if (!searched(j)) thr[j] = gs.start[j] <= 0 ? 0ull : ~0ull;
-  cl.sync();                                           // every CTA's eqc is complete
-  for (int j = 0; j < nb; ++j) {
-    if (!searched(j)) continue;                        // the same in every thread
+  const int r0 = min(n_loc, (int)threadIdx.x * run), r1 = min(n_loc, r0 + run);
+  for (int j = 0; __builtin_expect(shared_value, 0) && j < nb; ++j) {
+    if (target[j] < 0 || count[j] <= kCsList) continue;   // the same in every thread
     int before_cta = 0;                                // equal keys in earlier CTAs
     for (int r = 0; r < cta; ++r) before_cta += *cl.map_shared_rank(&eqc[j], r);
-    const int need = gs.start[j] - below[j] - before_cta;
+    const int need = target[j] - below[j] - before_cta;
     if (need < 0 || need >= eqc[j]) continue;          // another CTA holds it
-    const uint32_t kj = pre[j];
+    const uint32_t kj = low[j];
     int eq = 0;
     for (int n = r0; n < r1; ++n) eq += skey[n] == kj;
     int incl = eq;
@@ -558,20 +681,11 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
       const int t = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += t;
     }
+    __syncthreads();                                   // warp_tot is free
     if (lane == 31) warp_tot[w] = incl;
     __syncthreads();
-    if (w == 0) {
-      const int x = warp_tot[lane];
-      int inc = x;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-      }
-      warp_tot[lane] = inc - x;
-    }
-    __syncthreads();
-    const int before = warp_tot[w] + incl - eq;
+    const int wt = warp_tot[lane];
+    const int before = __reduce_add_sync(0xffffffffu, lane < w ? wt : 0) + incl - eq;
     if (need >= before && need < before + eq) {
       int seen = before;
       for (int n = r0; n < r1; ++n) {
@@ -584,14 +698,31 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
         ++seen;
       }
     }
-    __syncthreads();                                   // warp_tot is reused
   }
   cl.sync();                  // the boundary pairs have reached every CTA
-  for (int n = threadIdx.x; n < n_loc; n += kCsThreads) {
-    const unsigned long long kn = ((unsigned long long)skey[n] << 32) | (unsigned)(lo + n);
-    int passed = 0;
-    for (int j = 0; j < nb; ++j) passed += kn >= thr[j];
-    group_of[lo + n] = K - 1 - passed;
+  unsigned long long t4[4];                            // the first four, in registers
+#pragma unroll
+  for (int q = 0; q < 4; ++q) t4[q] = q < nb ? thr[q] : ~0ull;
+  const bool vec_out = (reinterpret_cast<uintptr_t>(group_of) & 15) == 0;
+  for (int i = threadIdx.x; i < n4; i += kCsThreads) {
+    const uint4 k4 = ckey4[i];
+    const uint32_t kk[4] = {k4.x, k4.y, k4.z, k4.w};
+    int g[4] = {nb, nb, nb, nb};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const unsigned long long kn = ((unsigned long long)kk[e] << 32) | (unsigned)(lo + 4 * i + e);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g[e] -= kn >= t4[q];
+      for (int j = 4; j < nb; ++j) g[e] -= kn >= thr[j];
+    }
+    int32_t *dst = group_of + lo + 4 * i;
+    if (vec_out && 4 * i + 3 < n_loc) {
+      *reinterpret_cast<int4 *>(dst) = make_int4(g[0], g[1], g[2], g[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (4 * i + e < n_loc) dst[e] = g[e];
+    }
   }
 }
 
@@ -769,6 +900,7 @@ namespace {
 // Opts the cluster kernel in to its shared memory on the current device and
 // checks that one cluster of kCsCtas such CTAs can be resident; otherwise the
 // partition takes the radix-sort path.  Resolved once per device.
+template <int kPer>
 bool cluster_select_ready() {
   static std::atomic<int> state[64];            // 0 unknown, 1 ready, 2 unavailable
   int dev = 0;
@@ -776,15 +908,16 @@ bool cluster_select_ready() {
   int st = state[dev].load();
   if (st == 0) {
     st = 2;
-    const int smem = kCsMaxChunk * (int)sizeof(uint32_t);
-    if (cudaFuncSetAttribute(cluster_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) == cudaSuccess) {
+    const int smem = kCsMaxChunk * (int)sizeof(uint32_t) + kCsFixedBytes;
+    if (cudaFuncSetAttribute(cluster_select_kernel<kPer>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(kCsCtas);
       cfg.blockDim = dim3(kCsThreads);
       cfg.dynamicSmemBytes = smem;
       int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, cluster_select_kernel, &cfg) == cudaSuccess &&
+      if (cudaOccupancyMaxActiveClusters(&clusters, cluster_select_kernel<kPer>, &cfg) ==
+              cudaSuccess &&
           clusters >= 1)
         st = 1;
     }
@@ -890,11 +1023,15 @@ extern "C" int hsa_partition(const float *stat, int N, int T, const int *budgets
                group_of, err);
     return launch_status();
   }
-  if (N <= kCsMaxN && cluster_select_ready()) {
+  // 2048 bins while they hold few keys each, 4096 for larger layers (a lognormal
+  // statistic of 200000 tokens would need a second pass with 2048: 35 us against 24).
+  const bool fine = N > kCsFineN;
+  if (N <= kCsMaxN && (fine ? cluster_select_ready<4>() : cluster_select_ready<2>())) {
     const int chunk = (((N + kCsCtas - 1) / kCsCtas) + 3) & ~3;   // keys per CTA, whole uint4
     count_launches(1);
-    cluster_select_kernel<<<kCsCtas, kCsThreads, (size_t)chunk * sizeof(uint32_t), s>>>(
-        stat, N, chunk, K, gs, group_of, err);
+    launch_pdl(fine ? cluster_select_kernel<4> : cluster_select_kernel<2>, dim3(kCsCtas),
+               dim3(kCsThreads), (size_t)chunk * sizeof(uint32_t) + kCsFixedBytes, s, stat, N,
+               chunk, K, gs, group_of, err);
     return launch_status();
   }
   // The scan's cluster is one CTA where a cluster of 8 cannot be resident.
