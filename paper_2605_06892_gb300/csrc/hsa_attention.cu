@@ -8,7 +8,7 @@
 // group, which is active at every iteration and so needs no cache.  Warp roles:
 //   warp 0      TMA producer: K and V tiles of the head, 128-byte swizzled,
 //               into a ring of shared-memory slots (rows >= N are zero-filled).
-//   warp 1      tensor-core issuer (lane 0 issues, the warp walks the
+//   warp 1      tensor-core issuer (one lane issues, the warp walks the
 //               schedule): S_t = Q_t K^T into TMEM and O_t += P_t V from TMEM
 //               P and shared V, tcgen05.mma kind::f16.
 //   warp 2      K/V watcher: waits for the K/V tiles to land, hands them to
@@ -156,28 +156,40 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int b_mn_major) 
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One lane of the warp: 1 in it, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(r));
+  return r;
+}
+
+// The MMAs and commits are issued by the lane with lead != 0, but every lane of
+// the issuing warp runs the code around them (see the issuer).
 __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t id,
-                                       uint32_t acc) {
+                                       uint32_t acc, uint32_t lead) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(id), "r"(acc)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"(acc), "r"(lead)
       : "memory");
 }
 
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t id,
-                                       uint32_t acc) {
+                                       uint32_t acc, uint32_t lead) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-      "r"(a_tmem), "l"(b), "r"(id), "r"(acc)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a_tmem), "l"(b), "r"(id), "r"(acc), "r"(lead)
       : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint64_t *b) {
+__device__ __forceinline__ void mma_commit(uint64_t *b, uint32_t lead) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_addr(b))
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          smem_addr(b)),
+      "r"(lead)
       : "memory");
 }
 
@@ -452,7 +464,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the same in every lane, and read from one: branches on it and what is
+  // computed under them stay uniform for the compiler
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int lane = threadIdx.x & 31;
   const CtaWork wk = cta_work(blockIdx.x, a.n_qblocks, a.n_whole, a.pieces, a.n_kv_tiles);
   const int h = wk.head;
   const int row0 = wk.row0;
@@ -555,7 +570,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = tmem_base_sh;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base_sh, 0);
 
   // The warpgroups' code paths never rejoin below: each ends with its own
   // teardown on named barrier 1, so each path is compiled for its own
@@ -585,7 +600,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       } else if (warp == 1) {
       // ------------------------------------------------ MMA issuer
       // The whole warp walks the schedule so that it can take part in the
-      // named-barrier hand-offs; lane 0 issues the MMAs and commits.  The
+      // named-barrier hand-offs; one lane issues the MMAs and commits.  The
       // tensor pipe takes a new MMA only about when it starts it, so every
       // pause of the issuing thread between MMAs idles the tensor core.  An
       // mbarrier test on this path costs about a hundred clocks while an S
@@ -601,7 +616,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       // per load of the abort flag), so after an abort it keeps issuing, over
       // whatever the ring and the TMEM hold, until the schedule ends; the
       // kernel then returns with the error recorded.
-      const bool leader = lane == 0;
+      // Every lane computes the addresses and descriptors of the MMAs, in code
+      // without divergence, and only the instruction itself is predicated to
+      // one lane.  The values are then uniform to the compiler; under a branch
+      // on the lane each MMA first had to move its operands there, in issue
+      // slots that two softmax warps of the same scheduler compete for, and the
+      // tensor core waited for them: D = 64, whose MMAs are half as long, went
+      // from 1269 to 1505 TFLOP/s (24 heads, N = 32760), the LTX layer from 980
+      // to 1132.  D = 128 is bound by the MMAs (1990 -> 1995).
+      const uint32_t lead = elect_one();
       constexpr uint32_t kIdS = idesc_bf16(kBM, kBN, 0);
       constexpr uint32_t kIdO = idesc_bf16(kBM, D, 1);
       const uint32_t q_base = smem_addr(sQ);
@@ -620,7 +643,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
           const uint32_t off = ((k >> 2) * (kBM * 128) + (k & 3) * 32) >> 4;
-          mma_ss(ts, dq + off, dk + off, kIdS, k > 0);
+          mma_ss(ts, dq + off, dk + off, kIdS, k > 0, lead);
         }
       };
       // O_t += P_t V: P in TMEM (bf16 pairs in the S_t columns), V MN-major.
@@ -629,7 +652,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const uint32_t to = tmem + C::kOCol0 + D * t, tp = tmem + 128 * t;
 #pragma unroll
         for (int k = 0; k < kBN / 16; ++k)
-          mma_ts(to, tp + 8 * k, dv + ((k * 2048) >> 4), kIdO, (acc || k > 0) ? 1u : 0u);
+          mma_ts(to, tp + 8 * k, dv + ((k * 2048) >> 4), kIdO, (acc || k > 0) ? 1u : 0u, lead);
       };
       auto p_ready = [&](int t) {
         named_barrier_sync(kBarP0 + t, kMeetP);
@@ -638,31 +661,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       if constexpr (!C::kThreeS) {
         named_barrier_sync(kBarK0, 64);             // K_0 has landed
         fence_after();
-        if (leader) {
-          issue_s(0, 0);
-          mma_commit(&bar_s[0]);
-          issue_s(1, 0);
-          mma_commit(&bar_s[1]);
-        }
+        issue_s(0, 0);
+        mma_commit(&bar_s[0], lead);
+        issue_s(1, 0);
+        mma_commit(&bar_s[1], lead);
         for (int j = 0; j < nT; ++j) {
           const int Lv = 2 * j + 1, Lk = 2 * j + 2;
           const bool more = j + 1 < nT;
           p_ready(0);                               // P_0(j); V_j and K_(j+1) landed
-          const bool go = leader;
-          if (go) {
-            issue_o(0, Lv, j > 0);
-            if (more) {
-              issue_s(0, Lk);
-              mma_commit(&bar_s[0]);
-            }
+          issue_o(0, Lv, j > 0);
+          if (more) {
+            issue_s(0, Lk);
+            mma_commit(&bar_s[0], lead);
           }
           p_ready(1);
-          if (go) {
-            issue_o(1, Lv, j > 0);
-            if (more) {
-              issue_s(1, Lk);
-              mma_commit(&bar_s[1]);
-            }
+          issue_o(1, Lv, j > 0);
+          if (more) {
+            issue_s(1, Lk);
+            mma_commit(&bar_s[1], lead);
           }
         }
       } else {
@@ -680,47 +696,38 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
           for (int k = 0; k < D / 16; ++k) {
             const uint32_t off = ((k >> 2) * (kBM * 128) + (k & 3) * 32) >> 4;
-            mma_ss(ts, dq + off, dk + off, kIdS, k > 0);
+            mma_ss(ts, dq + off, dk + off, kIdS, k > 0, lead);
           }
-          mma_commit(&bar_s[2 * t + (j & 1)]);
+          mma_commit(&bar_s[2 * t + (j & 1)], lead);
         };
         auto issue_o3 = [&](int t, int j) {
           const uint64_t dv = dv0 + ((2 * j + 1) % C::kStages) * kTile16;
           const uint32_t to = tmem + C::kOCol0 + D * t, tp = tmem + 128 * ((2 * j + t) % 3);
 #pragma unroll
           for (int k = 0; k < kBN / 16; ++k)
-            mma_ts(to, tp + 8 * k, dv + ((k * 2048) >> 4), kIdO, (j > 0 || k > 0) ? 1u : 0u);
+            mma_ts(to, tp + 8 * k, dv + ((k * 2048) >> 4), kIdO, (j > 0 || k > 0) ? 1u : 0u, lead);
         };
         named_barrier_sync(kBarK0, 64);             // K_0 (and K_1) have landed
         fence_after();
-        if (leader) {
-          issue_s3(0, 0);
-          issue_s3(1, 0);
-          if (nT > 1) issue_s3(0, 1);
-        }
+        issue_s3(0, 0);
+        issue_s3(1, 0);
+        if (nT > 1) issue_s3(0, 1);
         for (int j = 0; j < nT; ++j) {
           p_ready(0);                               // P_0(j); V_j and K_(j+1) landed
-          const bool go = leader;
-          if (go) {
-            issue_o3(0, j);
-            if (j + 1 < nT) issue_s3(1, j + 1);
-          }
+          issue_o3(0, j);
+          if (j + 1 < nT) issue_s3(1, j + 1);
           p_ready(1);                               // P_1(j); K_(j+2) landed
-          if (go) {
-            issue_o3(1, j);
-            if (j + 2 < nT)
-              issue_s3(0, j + 2);
-            else if (j + 2 == nT)
-              mma_commit(&bar_s[(j + 2) & 1]);      // O_1(j) done, for the last tile's rescale
-          }
+          issue_o3(1, j);
+          if (j + 2 < nT)
+            issue_s3(0, j + 2);
+          else if (j + 2 == nT)
+            mma_commit(&bar_s[(j + 2) & 1], lead);  // O_1(j) done, for the last tile's rescale
         }
       }
-      if (leader) {
-        // Completes once every MMA issued above has finished (also on
-        // abort), so TMEM is quiet before it is freed.
-        mma_commit(&bar_o);
-        mbar_wait(&bar_o, 0, &abort_flag, a.err, false);
-      }
+      // Completes once every MMA issued above has finished (also on abort), so
+      // TMEM is quiet before it is freed.
+      mma_commit(&bar_o, lead);
+      mbar_wait(&bar_o, 0, &abort_flag, a.err, false);
       __syncwarp();
     } else if (warp == 2) {
       // ------------------------------------------------ K/V watcher
