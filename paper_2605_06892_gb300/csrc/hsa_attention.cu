@@ -14,7 +14,8 @@
 //   warp 2      K/V watcher: waits for the K/V tiles to land, hands them to
 //               the issuer at the P meetings, and gives ring slots back to
 //               the producer.
-//   warp 3      idle (it completes the first warpgroup).
+//   warp 3      S watcher: waits for each S tile to complete and meets its
+//               softmax group.
 //   warps 4-7   softmax of Q tile 0, warps 8-11 softmax of Q tile 1: each
 //               thread owns one query row (its TMEM lane; a warp may only
 //               reach the lane quarter warp%4), reads its S row,
@@ -280,6 +281,10 @@ constexpr int kBarTeardown = 1;
 constexpr int kBarP0 = 2;
 constexpr int kBarK0 = 4;
 constexpr int kMeetP = kBM + 64;   // threads at a P meeting
+// kBarS0 + t: S of Q tile t is complete, for key tile j (its 128 softmax threads
+// and the S watcher meet).
+constexpr int kBarS0 = 5;
+constexpr int kMeetS = kBM + 32;
 
 template <int D>
 struct TcCfg {
@@ -793,6 +798,25 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           named_barrier_sync(kBarP0 + 1, kMeetP);
         }
       }
+    } else if (warp == 3) {
+      // ------------------------------------------------ S watcher
+      // An mbarrier test by a softmax warp takes about 300 clocks while the S
+      // groups' operand reads fill the shared-memory bandwidth, on a completed
+      // phase too; a named barrier takes a tenth of that.  So this warp makes
+      // the (bounded) test, ahead of need where the scores are computed ahead,
+      // and meets the softmax group.  It meets even after a failed wait.  24 x
+      // 64, N = 32760: 1508 -> 1595 TFLOP/s; Wan-1.3B shape 2005 -> 2027.
+      bool live = true;
+      for (int j = 0; j < nT; ++j) {
+#pragma unroll
+        for (int t = 0; t < kQT; ++t) {
+          uint64_t *b = C::kThreeS ? &bar_s[2 * t + (j & 1)] : &bar_s[t];
+          const uint32_t par = C::kThreeS ? (j >> 1) & 1 : j & 1;
+          if (live) live = __all_sync(0xffffffffu, mbar_wait(b, par, &abort_flag, a.err));
+          fence_before();
+          named_barrier_sync(kBarS0 + t, kMeetS);
+        }
+      }
     }
     fence_before();
     named_barrier_sync(kBarTeardown, kTcThreads);
@@ -813,50 +837,45 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const uint32_t tO = tmem + lane_off + C::kOCol0 + D * t;
     const float sl2 = a.scale_log2;
     float m_run = -INFINITY, l_run = 0.f;
-    // `ok` stays warp-uniform (the tile code votes across the warp).  After
-    // a failed wait the warp does no more work but still meets the issuer for
-    // every P, so the issuing warp's named-barrier syncs all complete.
-    // Meeting (rather than arriving) costs nothing: S_t(j+1) is issued only
-    // after the issuer has passed this meeting for P_t(j).
-    bool ok = true;
+    // The S watcher and the issuer are met for every key tile whatever happens,
+    // so all their syncs complete: after a failed wait the tiles are formed from
+    // whatever TMEM holds, and the abort flag, read before the rows are stored,
+    // keeps them from being written.  Meeting the issuer (rather than arriving)
+    // costs nothing: S_t(j+1) is issued only after the issuer has passed this
+    // meeting for P_t(j).
     for (int j = 0; j < nT; ++j) {
-      if constexpr (!C::kThreeS) {
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar_s[t], j & 1, &abort_flag, a.err));
-      } else {
-        if (ok)
-          ok = __all_sync(0xffffffffu, mbar_wait(&bar_s[2 * t + (j & 1)], (j >> 1) & 1,
-                                                 &abort_flag, a.err));
-      }
-      if (ok) {
+      named_barrier_sync(kBarS0 + t, kMeetS);      // S_t(j) is complete
+      fence_after();
+      const int jg = key_tile(j);                // keys of this tile that exist
+      const int valid = jg < a.tiles1 ? a.rows1 - jg * kBN : a.rows2 - (jg - a.tiles1) * kBN;
+      // three S buffers (D = 64): S_t(j) is the (2j + t)-th S MMA
+      const uint32_t tSj = C::kThreeS ? tmem + lane_off + 128 * ((2 * j + t) % 3) : tS;
+      // O_t(j-1) has completed once an MMA issued after it has.  With two
+      // S buffers that is S_t(j), complete already.  With three, S_t(j) is
+      // issued before O_t(j-1): wait for S_1(j) (Q tile 0) or S_0(j+1) (Q
+      // tile 1; at the last key tile the issuer commits that barrier with
+      // no MMA).  Neither barrier can complete again before this warp's
+      // next meeting.  Needed only on the exact path's rescale, so rare.
+      auto o_idle = [&]() -> bool {
+        if constexpr (!C::kThreeS) return true;
+        uint64_t *b = t == 0 ? &bar_s[2 + (j & 1)] : &bar_s[(j + 1) & 1];
+        const uint32_t par = t == 0 ? (j >> 1) & 1 : ((j + 1) >> 1) & 1;
+        const bool idle = __all_sync(0xffffffffu, mbar_wait(b, par, &abort_flag, a.err));
         fence_after();
-        const int jg = key_tile(j);                // keys of this tile that exist
-        const int valid = jg < a.tiles1 ? a.rows1 - jg * kBN : a.rows2 - (jg - a.tiles1) * kBN;
-        // three S buffers (D = 64): S_t(j) is the (2j + t)-th S MMA
-        const uint32_t tSj = C::kThreeS ? tmem + lane_off + 128 * ((2 * j + t) % 3) : tS;
-        // O_t(j-1) has completed once an MMA issued after it has.  With two
-        // S buffers that is S_t(j), complete already.  With three, S_t(j) is
-        // issued before O_t(j-1): wait for S_1(j) (Q tile 0) or S_0(j+1) (Q
-        // tile 1; at the last key tile the issuer commits that barrier with
-        // no MMA).  Neither barrier can complete again before this warp's
-        // next meeting.  Needed only on the exact path's rescale, so rare.
-        auto o_idle = [&]() -> bool {
-          if constexpr (!C::kThreeS) return true;
-          uint64_t *b = t == 0 ? &bar_s[2 + (j & 1)] : &bar_s[(j + 1) & 1];
-          const uint32_t par = t == 0 ? (j >> 1) & 1 : ((j + 1) >> 1) & 1;
-          const bool idle = __all_sync(0xffffffffu, mbar_wait(b, par, &abort_flag, a.err));
-          fence_after();
-          return idle;
-        };
-        if (valid >= kBN)
-          softmax_tile<D, false>(tSj, tO, valid, j == 0, sl2, m_run, l_run, o_idle);
-        else
-          softmax_tile<D, true>(tSj, tO, valid, j == 0, sl2, m_run, l_run, o_idle);
-        tmem_wait_st();
-      }
+        return idle;
+      };
+      if (valid >= kBN)
+        softmax_tile<D, false>(tSj, tO, valid, j == 0, sl2, m_run, l_run, o_idle);
+      else
+        softmax_tile<D, true>(tSj, tO, valid, j == 0, sl2, m_run, l_run, o_idle);
+      tmem_wait_st();
       fence_before();
       named_barrier_sync(kBarP0 + t, kMeetP);
     }
-    if (ok && wk.piece >= 0 && mbar_wait(&bar_o, 0, &abort_flag, a.err)) {
+    // warp-uniform: the loads below span the warp
+    bool ok = __all_sync(0xffffffffu, mbar_wait(&bar_o, 0, &abort_flag, a.err));
+    ok = !__any_sync(0xffffffffu, abort_flag != 0) && ok;
+    if (ok && wk.piece >= 0) {
       // Piece of a split unit: unnormalised O, maximum and sum, for the combine.
       fence_after();
       const int prow = t * kBM + r;
@@ -874,7 +893,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       }
       reinterpret_cast<float2 *>(a.ws_ml)[(size_t)wk.piece * (kQT * kBM) + prow] =
           make_float2(m_run, l_run);
-    } else if (ok && mbar_wait(&bar_o, 0, &abort_flag, a.err)) {
+    } else if (ok) {
       fence_after();
       const int grow = row0 + t * kBM + r;
       const float inv = 1.f / l_run;
