@@ -447,17 +447,82 @@ __device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, int valid
   l_run += exp_store_tile(tS, r, sl2, m_run);
 }
 
+// Stores 32 finished rows of a unit (r0 .. r0+31 of its kQT*kBM; this lane holds
+// row r0 + lane in TMEM columns tO ..), or of a piece of a split unit
+// (unnormalised O, maximum and sum, for the combine), by way of `stage`, 32 * D
+// floats of the warp's own.  A lane's row there is a run of 16-byte vectors, their
+// order turned by the row so that the 8 lanes of a quarter-warp use distinct banks.
+// A lane that stores its own row touches 32 lines per instruction: 2000 clocks per
+// unit at D = 64, 4000 for a piece or at D = 128, on the one path to the L1.
+template <int D>
+__device__ __forceinline__ void store_rows(const TcArgs &a, const CtaWork &wk, int r0, int lane,
+                                           uint32_t tO, float m_run, float l_run,
+                                           uint8_t *stage) {
+  const bool piece = wk.piece >= 0;
+  const float inv = 1.f / l_run;
+  uint4 *st = reinterpret_cast<uint4 *>(stage);
+  if (piece) {
+    constexpr int kV = D / 4;                      // vectors per row
+#pragma unroll
+    for (int c = 0; c < D / 32; ++c) {
+      uint32_t o[32];
+      tmem_ld32(tO + 32 * c, o);
+      tmem_wait_ld();
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+        st[lane * kV + (8 * c + (v ^ (lane & 7)))] =
+            make_uint4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
+    }
+    __syncwarp();
+    uint4 *dst = reinterpret_cast<uint4 *>(a.ws_o) +
+                 ((size_t)wk.piece * (kQT * kBM) + r0) * kV;
+#pragma unroll 8
+    for (int i = 0; i < kV; ++i) {
+      const int e = 32 * i + lane, row = e / kV, v = e % kV;
+      dst[e] = st[row * kV + ((v & ~7) | ((v & 7) ^ (row & 7)))];
+    }
+    reinterpret_cast<float2 *>(a.ws_ml)[(size_t)wk.piece * (kQT * kBM) + r0 + lane] =
+        make_float2(m_run, l_run);
+    return;
+  }
+  constexpr int kV = D / 8;
+#pragma unroll
+  for (int c = 0; c < D / 32; ++c) {
+    uint32_t o[32];
+    tmem_ld32(tO + 32 * c, o);
+    tmem_wait_ld();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      uint32_t pk[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        pk[i] = pack_bf16(__uint_as_float(o[8 * v + 2 * i]) * inv,
+                          __uint_as_float(o[8 * v + 2 * i + 1]) * inv);
+      const int u = 4 * c + v;                     // vector of the row
+      st[lane * kV + ((u & ~7) | ((u & 7) ^ (lane & 7)))] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+  }
+  __syncwarp();
+  uint64_t pol;                 // the output rows are written once: evict first
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+#pragma unroll
+  for (int i = 0; i < kV; ++i) {
+    const int e = 32 * i + lane, row = e / kV, v = e % kV;
+    const int grow = wk.row0 + r0 + row;
+    const uint4 x = st[row * kV + ((v & ~7) | ((v & 7) ^ (row & 7)))];
+    if (grow < a.n_active)
+      asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(
+                       a.out + ((size_t)grow * a.H + wk.head) * D + 8 * v),
+                   "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "l"(pol)
+                   : "memory");
+  }
+}
+
 template <int D>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_k2, const __grid_constant__ CUtensorMap tm_v2,
                const TcArgs a) {
-  // Launched with programmatic dependent launch: wait for the kernels before
-  // this one in the stream (the KV scatter writes the keys read below).  The
-  // blocks of the last wave let the next kernel start launching onto the SMs
-  // they free; no block of this grid is still waiting for an SM by then.
-  pdl_wait();
-  if (blockIdx.x + (unsigned)a.wave >= gridDim.x) pdl_trigger();
   using C = TcCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -501,7 +566,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       tma_load_2d(dst + c * (kBN * 128), map, &bar_full[slot], h * D + c * 64, y);
   };
   const int withheld = a.inject_stall == 1 ? 1 : -1;   // test hook: V of tile 0 never loads
-  const int n_pre = min(C::kStages, 2 * nT);          // loads issued before the Q tile
+  const int n_pre = min(3, 2 * nT);                   // loads issued before the Q tile: K_0 V_0 K_1
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
       mbar_init(&bar_full[s], 1);
@@ -512,10 +577,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // The first ring's worth of K/V tiles load while the CTA loads its query
-    // rows below.
-    for (int L = 0; L < n_pre; ++L)
-      if (L != withheld) load_kv(L);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -524,6 +585,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // Launched with programmatic dependent launch: up to here the block touches
+  // only its own SM, and runs beside the end of the kernel before it; wait for
+  // that kernel and those before it (the KV scatter writes the keys read below).
+  // The blocks of the last wave let the next kernel start launching onto the SMs
+  // they free; no block of this grid is still waiting for an SM by then.
+  pdl_wait();
+  if (blockIdx.x + (unsigned)a.wave >= gridDim.x) pdl_trigger();
+  // The first key tiles load while the CTA loads its query rows below, and no
+  // more than the first MMAs need: a whole ring's worth on every SM at once held
+  // the query rows up for 2000 clocks.
+  if (threadIdx.x == 0)
+    for (int L = 0; L < n_pre; ++L)
+      if (L != withheld) load_kv(L);
 
   // ---- query rows, by index, into the two swizzled Q tiles (all threads)
   // Each thread first reads the indices of all its rows, then issues all its
@@ -875,50 +949,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // warp-uniform: the loads below span the warp
     bool ok = __all_sync(0xffffffffu, mbar_wait(&bar_o, 0, &abort_flag, a.err));
     ok = !__any_sync(0xffffffffu, abort_flag != 0) && ok;
-    if (ok && wk.piece >= 0) {
-      // Piece of a split unit: unnormalised O, maximum and sum, for the combine.
+    // Every MMA has completed, so the ring's memory is free: each warp turns its
+    // 32 rows around in its own part of it, so that neighbouring lanes store
+    // neighbouring 16-byte vectors.
+    if (ok) {
       fence_after();
-      const int prow = t * kBM + r;
-      float *po = a.ws_o + ((size_t)wk.piece * (kQT * kBM) + prow) * D;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t o[32];
-        tmem_ld32(tO + 32 * c, o);
-        tmem_wait_ld();
-        float4 *d4 = reinterpret_cast<float4 *>(po + 32 * c);
-#pragma unroll
-        for (int v = 0; v < 8; ++v)
-          d4[v] = make_float4(__uint_as_float(o[4 * v]), __uint_as_float(o[4 * v + 1]),
-                              __uint_as_float(o[4 * v + 2]), __uint_as_float(o[4 * v + 3]));
-      }
-      reinterpret_cast<float2 *>(a.ws_ml)[(size_t)wk.piece * (kQT * kBM) + prow] =
-          make_float2(m_run, l_run);
-    } else if (ok) {
-      fence_after();
-      const int grow = row0 + t * kBM + r;
-      const float inv = 1.f / l_run;
-      __nv_bfloat16 *dst = a.out + ((size_t)grow * a.H + h) * D;
-#pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t o[32];
-        tmem_ld32(tO + 32 * c, o);
-        tmem_wait_ld();
-        uint32_t pk[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          pk[i] = pack_bf16(__uint_as_float(o[2 * i]) * inv, __uint_as_float(o[2 * i + 1]) * inv);
-        if (grow < a.n_active) {
-          uint64_t pol;                 // the output rows are written once: evict first
-          asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-#pragma unroll
-          for (int v = 0; v < 4; ++v)
-            asm volatile("st.global.L2::cache_hint.v4.u32 [%0], {%1,%2,%3,%4}, %5;" ::"l"(
-                             dst + 32 * c + 8 * v),
-                         "r"(pk[4 * v]), "r"(pk[4 * v + 1]), "r"(pk[4 * v + 2]),
-                         "r"(pk[4 * v + 3]), "l"(pol)
-                         : "memory");
-        }
-      }
+      store_rows<D>(a, wk, t * kBM + wq * 32, lane, tO, m_run, l_run,
+                    sKV + (warp - 4) * (32 * D * 4));
     }
     fence_before();
     named_barrier_sync(kBarTeardown, kTcThreads);
@@ -927,9 +964,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 
 // ------------------------------------------------------ split-unit combine
 //
-// One warp per (tail unit, row): merge the unit's key-range pieces,
-// O = sum_p 2^(m_p - M) O_p / sum_p 2^(m_p - M) l_p with M = max_p m_p, and
-// store the bf16 row.  Lanes stride over D, so every access is coalesced.
+// D/4 lanes per (tail unit, row), four dimensions each: merge the unit's
+// key-range pieces, O = sum_p 2^(m_p - M) O_p / sum_p 2^(m_p - M) l_p with M =
+// max_p m_p, and store the bf16 row.  Bound by latency (the pieces are in L2), so
+// lane p of the row loads (m, l) of piece p and the weights go around by
+// shuffles, then all pieces' vectors load at once: two round trips to memory.
 template <int D>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const float *__restrict__ ws_o, const float *__restrict__ ws_ml, int n_tail,
@@ -937,32 +976,43 @@ attn_combine_kernel(const float *__restrict__ ws_o, const float *__restrict__ ws
                     __nv_bfloat16 *__restrict__ out) {
   pdl_wait();
   pdl_trigger();
-  constexpr int kRows = kQT * kBM;
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  constexpr int kRows = kQT * kBM, kL = D / 4;     // lanes per row
+  const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) / kL);
+  const int sub = threadIdx.x % kL;
   const int u = wid / kRows, row = wid % kRows;
-  if (u >= n_tail) return;
+  if (u >= n_tail) return;                         // whole warps: kRows rows are whole warps
   const int unit = n_whole + u;
   const int head = unit / n_qblocks;
   const int grow = (unit % n_qblocks) * kRows + row;
-  if (grow >= n_active) return;
-  const float2 *ml = reinterpret_cast<const float2 *>(ws_ml);
+  const float2 *ml = reinterpret_cast<const float2 *>(ws_ml) + (size_t)u * pieces * kRows + row;
+  const float4 *o = reinterpret_cast<const float4 *>(ws_o) +
+                    ((size_t)u * pieces * kRows + row) * kL + sub;
   float M = -INFINITY;
-  for (int p = 0; p < pieces; ++p) M = fmaxf(M, ml[((size_t)u * pieces + p) * kRows + row].x);
-  float L = 0.f, acc[D / 32];
+  for (int p = sub; p < pieces; p += kL) M = fmaxf(M, ml[(size_t)p * kRows].x);
 #pragma unroll
-  for (int i = 0; i < D / 32; ++i) acc[i] = 0.f;
-  for (int p = 0; p < pieces; ++p) {
-    const size_t pr = ((size_t)u * pieces + p) * kRows + row;
-    const float2 v = ml[pr];
-    const float w = exp2f(v.x - M);
-    L = fmaf(w, v.y, L);
-#pragma unroll
-    for (int i = 0; i < D / 32; ++i) acc[i] = fmaf(w, ws_o[pr * D + lane + 32 * i], acc[i]);
+  for (int x = 1; x < kL; x <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
+  float L = 0.f;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int p0 = 0; p0 < pieces; p0 += kL) {
+    float2 v = make_float2(-INFINITY, 0.f);
+    if (p0 + sub < pieces) v = ml[(size_t)(p0 + sub) * kRows];
+    const float wl = exp2f(v.x - M);
+    const int np = min(kL, pieces - p0);
+#pragma unroll 8
+    for (int p = 0; p < np; ++p) {
+      const float4 x = o[(size_t)(p0 + p) * kRows * kL];
+      const float w = __shfl_sync(0xffffffffu, wl, p, kL);
+      L = fmaf(w, __shfl_sync(0xffffffffu, v.y, p, kL), L);
+      acc.x = fmaf(w, x.x, acc.x);
+      acc.y = fmaf(w, x.y, acc.y);
+      acc.z = fmaf(w, x.z, acc.z);
+      acc.w = fmaf(w, x.w, acc.w);
+    }
   }
+  if (grow >= n_active) return;
   const float inv = 1.f / L;
-  __nv_bfloat16 *dst = out + ((size_t)grow * H + head) * D;
-#pragma unroll
-  for (int i = 0; i < D / 32; ++i) dst[lane + 32 * i] = __float2bfloat16_rn(acc[i] * inv);
+  *reinterpret_cast<uint2 *>(out + ((size_t)grow * H + head) * D + 4 * sub) =
+      make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
 }
 
 // -------------------------------------------------------------- host side
@@ -1097,9 +1147,9 @@ int launch_tc(const void *q, const int32_t *q_idx, int n_active, const void *k_c
              mk2, mv2, a);
   if (cudaGetLastError() != cudaSuccess) return HSA_ERR_CUDA;
   if (pieces > 1) {
-    const long long warps = (long long)rem * (kQT * kBM);
+    const long long threads = (long long)rem * (kQT * kBM) * (D / 4);
     count_launches(1);
-    launch_pdl(attn_combine_kernel<D>, dim3((unsigned)((warps * 32 + 255) / 256)), dim3(256), 0,
+    launch_pdl(attn_combine_kernel<D>, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0,
                stream, (const float *)a.ws_o, (const float *)a.ws_ml, (int)rem, a.n_whole,
                pieces, a.n_qblocks, n_active, H, a.out);
   }
