@@ -21,10 +21,11 @@ namespace {
 constexpr int kThreads = 256;
 // 16-byte vectors each lane keeps in flight (measured on GB300 with an L2-
 // flushed size sweep: the gather reaches its best rate at 4, the scatter,
-// whose loads are contiguous, at 8; Euler holds two vectors per step).
+// whose loads are contiguous, at 8; Euler holds two vectors per step on long
+// rows, see hsa_cached_euler).
 constexpr int kGatherUnroll = 4;
 constexpr int kScatterUnroll = 8;
-constexpr int kEulerUnroll = 2;  // float4 positions per thread per pass (large N)
+constexpr int kEulerUnroll = 2;  // float4 positions per thread per pass (long rows, large N)
 
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
   uint4 v;
@@ -107,6 +108,23 @@ kv_scatter_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc,
   });
 }
 
+// pos[row], with a bad entry (only -1 means "no fresh row") reported and read as
+// -1.
+__device__ __forceinline__ int load_pos(const int32_t *__restrict__ pos, long long row,
+                                        int n_fresh_rows, unsigned *err) {
+  const int p = __ldg(pos + row);
+  if (p >= n_fresh_rows || p < -1) {
+    set_error(err, kErrIndex);
+    return -1;
+  }
+  return p;
+}
+
+__device__ __forceinline__ float4 euler_step(const float4 &v, float dsigma, const float4 &x) {
+  return make_float4(__fmaf_rn(v.x, dsigma, x.x), __fmaf_rn(v.y, dsigma, x.y),
+                     __fmaf_rn(v.z, dsigma, x.z), __fmaf_rn(v.w, dsigma, x.w));
+}
+
 // x[n] = fma(vhat[n], dsigma, x[n]) with vhat[n] refreshed from
 // v_fresh[pos[n]] when pos[n] >= 0.  Element-wise over the N*C/4 float4
 // vectors: each thread takes kU vectors a grid-stride apart.  The pos entries
@@ -116,7 +134,11 @@ kv_scatter_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc,
 // grid is the number of blocks resident at once (a single wave).  Measured on
 // GB300 with an L2-flushed size sweep: kU = 2 with the pos loads one pass
 // ahead reaches 0.85-1.0 of the HBM copy rate, kU = 4 (more registers, fewer
-// resident threads) 0.68-0.85.
+// resident threads) 0.68-0.85.  Rows below 16 vectors (C < 64) take one vector
+// per thread: half the tokens fresh, 3 layers in turn, 1048576 x 16 43.7 -> 42.2
+// us, 4000000 x 16 152.6 -> 147.7, 200000 x 48 26.3 -> 24.4; from 16 vectors on two
+// are the better (1048576 x 64 144.6 against 148.8, 262144 x 256 140.3 against
+// 146.8).
 // vec_shift = log2(C/4) when C/4 is a power of two, else -1 (division).
 // Small N uses one vector per thread (kU = 1) so that every SM has work.
 template <int kU>
@@ -128,14 +150,8 @@ __device__ __forceinline__ void load_pos_pass(const int32_t *__restrict__ pos, l
   for (int u = 0; u < kU; ++u) {
     const long long e = base + u * stride;
     p[u] = -1;
-    if (pos && e < total) {
-      const long long row = vec_shift >= 0 ? (e >> vec_shift) : e / vecs;
-      p[u] = __ldg(pos + row);
-      if (p[u] >= n_fresh_rows || p[u] < -1) {   // only -1 means "no fresh row"
-        set_error(err, kErrIndex);
-        p[u] = -1;
-      }
-    }
+    if (pos && e < total)
+      p[u] = load_pos(pos, vec_shift >= 0 ? (e >> vec_shift) : e / vecs, n_fresh_rows, err);
   }
 }
 
@@ -173,83 +189,63 @@ cached_euler_kernel(float4 *__restrict__ x, float4 *__restrict__ vhat,
       const long long e = base + u * stride;
       if (e < total) {
         if (p[u] >= 0) vhat[e] = vb[u];
-        float4 o;
-        o.x = __fmaf_rn(vb[u].x, dsigma, xb[u].x);
-        o.y = __fmaf_rn(vb[u].y, dsigma, xb[u].y);
-        o.z = __fmaf_rn(vb[u].z, dsigma, xb[u].z);
-        o.w = __fmaf_rn(vb[u].w, dsigma, xb[u].w);
-        x[e] = o;
+        x[e] = euler_step(vb[u], dsigma, xb[u]);
       }
     }
   }
 }
 
-// The cached Euler step fused with the velocity statistic (below), element-
-// wise like cached_euler_kernel, for C/4 a power of two <= 32: the C/4 lanes
-// of a token are consecutive lanes of one warp (passes start at a multiple of
-// 32), so the token's two L1 norms are reduced with log2(C/4) shuffles and the
-// token's first lane updates stat.  Every lane of a warp runs the same passes
-// (the shuffles span the warp).
-template <int kU>
-__global__ void __launch_bounds__(kThreads)
+// The cached Euler step fused with the velocity statistic (below) for rows of
+// up to 32 vectors (C <= 128): L = 2^lpr_log2 >= C/4 neighbouring lanes take a
+// token (those past its vectors idle), so its two L1 norms are reduced with
+// log2(L) shuffles and its first lane updates stat.  Every lane of a warp runs
+// the same passes (the shuffles span the warp).  HBM-bound, one vector per
+// thread keeps the registers at 32 and the SM full (2048 threads), which holds
+// more loads in flight than two vectors on half the threads.  Every token fresh,
+// 3 layers in turn: 1048576 x 16 68.6 -> 56.4 us (0.92 of the measured HBM rate),
+// 4000000 x 16 240 -> 208 (0.95), 1048576 x 64 244 -> 214 (0.95), 262144 x 128 125
+// -> 108 (0.93); 1048576 x 48, which took two tokens per lane group and pass
+// before, 270 -> 152 (1.00).
+__global__ void __launch_bounds__(kThreads, 8)
 euler_l1rel_elem_kernel(float4 *__restrict__ x, float4 *__restrict__ vhat,
                         const float4 *__restrict__ v_fresh, const int32_t *__restrict__ pos,
-                        long long total, int vecs, int vec_shift, float dsigma,
-                        int n_fresh_rows, float *__restrict__ stat, float weight, unsigned *err) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
+                        int N, int vecs, int lpr_log2, float dsigma, int n_fresh_rows,
+                        float *__restrict__ stat, float weight, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
-  long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  int pn[kU];
-  load_pos_pass<kU>(pos, base, stride, total, vecs, vec_shift, n_fresh_rows, err, pn);
-  for (; base - lane < total; base += stride * kU) {
-    int p[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) p[u] = pn[u];
-    load_pos_pass<kU>(pos, base + stride * kU, stride, total, vecs, vec_shift, n_fresh_rows,
-                      err, pn);
-    float4 vo[kU], vn[kU], xb[kU];
-    float st[kU];
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const long long e = base + u * stride;
-      st[u] = 0.f;
-      if (e < total) {
-        const long long row = e >> vec_shift;
-        const long long c = e - row * vecs;
-        xb[u] = x[e];
-        vo[u] = vhat[e];
-        vn[u] = p[u] >= 0 ? __ldg(v_fresh + (long long)p[u] * vecs + c) : vo[u];
-        if (p[u] >= 0 && (lane & (vecs - 1)) == 0) st[u] = stat[row];   // with the data
+  const int L = 1 << lpr_log2;
+  const int c = lane & (L - 1);
+  const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;   // tokens per pass
+  long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
+  int p = row < N ? load_pos(pos, row, n_fresh_rows, err) : -1;
+  for (; row - (lane >> lpr_log2) < N; row += step) {
+    const int p_next = row + step < N ? load_pos(pos, row + step, n_fresh_rows, err) : -1;
+    const bool in = row < N && c < vecs;
+    const bool first = p >= 0 && c == 0;               // p >= 0 only below N
+    const long long e = row * vecs + c;
+    float num = 0.f, den = 0.f, st = 0.f;
+    if (in) {
+      const float4 xv = x[e];
+      const float4 vo = vhat[e];
+      const float4 vn = p >= 0 ? __ldg(v_fresh + (long long)p * vecs + c) : vo;
+      if (first) st = stat[row];                       // with the data
+      if (p >= 0) {
+        num = fabsf(vn.x - vo.x) + fabsf(vn.y - vo.y) + fabsf(vn.z - vo.z) + fabsf(vn.w - vo.w);
+        den = fabsf(vn.x) + fabsf(vn.y) + fabsf(vn.z) + fabsf(vn.w);
+        vhat[e] = vn;
       }
+      x[e] = euler_step(vn, dsigma, xv);
     }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const long long e = base + u * stride;
-      float num = 0.f, den = 0.f;
-      if (e < total) {
-        if (p[u] >= 0) {
-          num = fabsf(vn[u].x - vo[u].x) + fabsf(vn[u].y - vo[u].y) + fabsf(vn[u].z - vo[u].z) +
-                fabsf(vn[u].w - vo[u].w);
-          den = fabsf(vn[u].x) + fabsf(vn[u].y) + fabsf(vn[u].z) + fabsf(vn[u].w);
-          vhat[e] = vn[u];
-        }
-        float4 o;
-        o.x = __fmaf_rn(vn[u].x, dsigma, xb[u].x);
-        o.y = __fmaf_rn(vn[u].y, dsigma, xb[u].y);
-        o.z = __fmaf_rn(vn[u].z, dsigma, xb[u].z);
-        o.w = __fmaf_rn(vn[u].w, dsigma, xb[u].w);
-        x[e] = o;
-      }
-      for (int o = 1; o < vecs; o <<= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
-      }
-      if (e < total && p[u] >= 0 && (lane & (vecs - 1)) == 0) {
-        const long long row = e >> vec_shift;
-        const float r = den > 0.f ? num / den : (num > 0.f ? 3.402823466e38f : 0.f);
-        stat[row] = fmaf(weight, r, st[u]);
-      }
+    for (int o = 1; o < L; o <<= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
     }
+    if (first) {
+      const float r = den > 0.f ? num / den : (num > 0.f ? 3.402823466e38f : 0.f);
+      stat[row] = fmaf(weight, r, st);
+    }
+    p = p_next;
   }
 }
 
@@ -258,9 +254,9 @@ euler_l1rel_elem_kernel(float4 *__restrict__ x, float4 *__restrict__ vhat,
 // row is v_{i-1}[n] and the fresh row v_i[n]; the kernel adds
 // weight * ||v_i - v_{i-1}||_1 / ||v_i||_1 to stat[n] (a zero denominator
 // counts 0 with a zero numerator, FLT_MAX otherwise), then refreshes the cache
-// and advances x exactly as cached_euler_kernel does.  This layout (for C/4
-// not a power of two, or above 32): a group of L lanes owns a token; the two
-// L1 norms are reduced across the group with shuffles.
+// and advances x exactly as cached_euler_kernel does.  This layout (for more
+// than 32 vectors per row): a group of L lanes owns a token; the two L1 norms
+// are reduced across the group with shuffles.
 constexpr int kL1relRows = 2;   // tokens per lane group per pass
 
 __global__ void __launch_bounds__(kThreads, 4)
@@ -268,6 +264,8 @@ euler_l1rel_kernel(float4 *__restrict__ x, float4 *__restrict__ vhat,
                    const float4 *__restrict__ v_fresh, const int32_t *__restrict__ pos,
                    int N, int vecs, int lpr_log2, float dsigma, int n_fresh_rows,
                    float *__restrict__ stat, float weight, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
   const int L = 1 << lpr_log2;
   const int lane = threadIdx.x & 31;
   const int sub = lane >> lpr_log2;
@@ -558,7 +556,8 @@ extern "C" int hsa_cached_euler(float *x, float *v_cache, const float *v_fresh,
   for (int sh = 0; sh < 31; ++sh)
     if ((1 << sh) == vecs) vec_shift = sh;
   const long long resident = (long long)sm_count() * 2048;     // threads
-  const int per = total >= (long long)kEulerUnroll * resident ? kEulerUnroll : 1;
+  const int per =
+      vecs >= 16 && total >= (long long)kEulerUnroll * resident ? kEulerUnroll : 1;
   long long blocks = (total + (long long)kThreads * per - 1) / ((long long)kThreads * per);
   const long long cap = per == kEulerUnroll ? resident_blocks<cached_euler_kernel<kEulerUnroll>>()
                                             : resident_blocks<cached_euler_kernel<1>>();
@@ -587,36 +586,21 @@ extern "C" int hsa_cached_euler_l1rel(float *x, float *v_cache, const float *v_f
   unsigned *err = device_error_word();
   if (!err) return HSA_ERR_CUDA;
   const int vecs = C / 4;
-  int vec_shift = -1;
-  for (int sh = 0; sh <= 5; ++sh)
-    if ((1 << sh) == vecs) vec_shift = sh;
-  if (vec_shift >= 0) {
-    // element-wise: C/4 a power of two, at most 32 (a token within one warp)
-    const long long total = (long long)N * vecs;
-    const long long resident = (long long)sm_count() * 2048;     // threads
-    const int per = total >= (long long)kEulerUnroll * resident ? kEulerUnroll : 1;
-    long long blocks = (total + (long long)kThreads * per - 1) / ((long long)kThreads * per);
-    const long long cap = per == kEulerUnroll
-                              ? resident_blocks<euler_l1rel_elem_kernel<kEulerUnroll>>()
-                              : resident_blocks<euler_l1rel_elem_kernel<1>>();
-    if (blocks > cap) blocks = cap;
-    count_launches(1);
-    if (per == kEulerUnroll)
-      euler_l1rel_elem_kernel<kEulerUnroll><<<(int)blocks, kThreads, 0, (cudaStream_t)stream>>>(
-          (float4 *)x, (float4 *)v_cache, (const float4 *)v_fresh, pos, total, vecs, vec_shift,
-          dsigma, n_fresh, stat, weight, err);
-    else
-      euler_l1rel_elem_kernel<1><<<(int)blocks, kThreads, 0, (cudaStream_t)stream>>>(
-          (float4 *)x, (float4 *)v_cache, (const float4 *)v_fresh, pos, total, vecs, vec_shift,
-          dsigma, n_fresh, stat, weight, err);
-    return launch_status();
-  }
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  euler_l1rel_kernel<<<grid_for(((long long)N + kL1relRows - 1) / kL1relRows, L), kThreads, 0,
-                       (cudaStream_t)stream>>>(
-      (float4 *)x, (float4 *)v_cache, (const float4 *)v_fresh, pos, N, vecs, log2i(L), dsigma,
-      n_fresh, stat, weight, err);
+  if (vecs <= 32) {
+    long long blocks = (((long long)N << log2i(L)) + kThreads - 1) / kThreads;
+    const long long cap = resident_blocks<euler_l1rel_elem_kernel>();
+    if (blocks > cap) blocks = cap;
+    launch_pdl(euler_l1rel_elem_kernel, dim3((unsigned)blocks), dim3(kThreads), 0,
+               (cudaStream_t)stream, (float4 *)x, (float4 *)v_cache, (const float4 *)v_fresh, pos,
+               N, vecs, log2i(L), dsigma, n_fresh, stat, weight, err);
+    return launch_status();
+  }
+  launch_pdl(euler_l1rel_kernel,
+             dim3((unsigned)grid_for(((long long)N + kL1relRows - 1) / kL1relRows, L)),
+             dim3(kThreads), 0, (cudaStream_t)stream, (float4 *)x, (float4 *)v_cache,
+             (const float4 *)v_fresh, pos, N, vecs, log2i(L), dsigma, n_fresh, stat, weight, err);
   return launch_status();
 }
 
