@@ -25,6 +25,10 @@ constexpr int kThreads = 256;
 // rows, see hsa_cached_euler).
 constexpr int kGatherUnroll = 4;
 constexpr int kScatterUnroll = 8;
+// The rotation in place is best at 6, the rotating scatter, which also holds the
+// table's vectors and two row pointers, at 4.
+constexpr int kRopeUnroll = 6;
+constexpr int kRopeScatterUnroll = 4;
 constexpr int kEulerUnroll = 2;  // float4 positions per thread per pass (long rows, large N)
 
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
@@ -341,13 +345,13 @@ euler_l1rel_kernel(float4 *__restrict__ x, float4 *__restrict__ vhat,
 // Rotary position embedding of the active rows (Sec. 2.3: the positional
 // frequencies are subsampled to A_i): row j of a token tensor is rotated by
 // the (cos, sin) table row of its token idx[j].  One 16-byte vector holds 8
-// bf16 values = 4 rotation pairs; pair (x0, x1) becomes
+// bf16 values = 4 rotation pairs, t0 and t1 their (c, s); pair (x0, x1) becomes
 // (fma(x0, c, -(x1 s)), fma(x0, s, x1 c)) in fp32, rounded to bf16.
-__device__ __forceinline__ uint4 rope8(uint4 v, const float4 *tab) {
+__device__ __forceinline__ uint4 rope8(uint4 v, const float4 &t0, const float4 &t1) {
   uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const float4 cs2 = __ldg(tab + (k >> 1));          // (c, s) of two pairs
+    const float4 &cs2 = k < 2 ? t0 : t1;
     const float c = (k & 1) ? cs2.z : cs2.x, s = (k & 1) ? cs2.w : cs2.y;
     const float x0 = __uint_as_float(w[k] << 16), x1 = __uint_as_float(w[k] & 0xffff0000u);
     const float y0 = __fmaf_rn(x0, c, -(x1 * s));
@@ -358,73 +362,101 @@ __device__ __forceinline__ uint4 rope8(uint4 v, const float4 *tab) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Rotates (or with `plain` copies) a row of `vecs` vectors from s to d, one lane
+// group of L lanes per row.  Vector v covers head 8v / D and pairs (8v mod D)/2 ..
+// +3.  kFixed: D/8 divides L, so a lane's vectors all sit at the same place of
+// their heads and its (c, s) are loaded once per row, with the row's vectors;
+// otherwise each vector loads its own.
+template <bool kFixed, int kU, class Load>
+__device__ __forceinline__ void rope_row(const uint4 *s, uint4 *d, const float4 *trow, int vecs,
+                                         int L, int sl, int D, bool plain, Load load) {
+  float4 t0 = make_float4(0.f, 0.f, 0.f, 0.f), t1 = t0;
+  if (kFixed && !plain) {
+    const int p = 2 * (sl & (D / 8 - 1));              // D/8 a power of two: it divides L
+    t0 = __ldg(trow + p);
+    t1 = __ldg(trow + p + 1);
+  }
+  for (int v0 = sl; v0 < vecs; v0 += kU * L) {
+    uint4 buf[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (v0 + u * L < vecs) buf[u] = load(s + v0 + u * L);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int v = v0 + u * L;
+      if (v >= vecs) continue;
+      if (!kFixed && !plain) {
+        const int p = 2 * (v % (D / 8));
+        t0 = __ldg(trow + p);
+        t1 = __ldg(trow + p + 1);
+      }
+      d[v] = plain ? buf[u] : rope8(buf[u], t0, t1);
+    }
+  }
+}
+
 // In-place rotation of rows j < n of x [n, H*D] (bf16): a lane group owns a
-// row; vector c covers head 8c / D and pairs ((8c) % D)/2 .. +3.
+// row; the index of its next row is loaded one row ahead.  HBM-bound; half of the
+// tokens, 3 layers in turn, against one vector in flight per lane and a remainder
+// by D for each: 32760 tokens x 12 x 128 24.8 -> 18.5 us (0.88 of the measured HBM
+// rate), 75600 x 40 x 128 158 -> 120 (0.99).
+template <bool kFixed>
 __global__ void __launch_bounds__(kThreads)
 rope_rows_kernel(uint4 *__restrict__ x, const int32_t *__restrict__ idx, int n, int vecs, int D,
                  const float4 *__restrict__ table, int N, int lpr_log2, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
   const int L = 1 << lpr_log2;
   const int lane = threadIdx.x & 31;
-  const int sub = lane >> lpr_log2, sl = lane & (L - 1);
-  const int rows_per_warp = 32 >> lpr_log2;
-  const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const int pairs = D / 2;
-  for (long long j = warp * rows_per_warp + sub; j < n; j += nwarps * rows_per_warp) {
-    const int t = __ldg(idx + j);
-    if (t < 0 || t >= N) {
+  const int sl = lane & (L - 1);
+  const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;
+  long long j = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
+  int t = j < n ? __ldg(idx + j) : 0;
+  for (; j < n; j += step) {
+    const int t_next = j + step < n ? __ldg(idx + j + step) : 0;
+    if (t < 0 || t >= N)
       set_error(err, kErrIndex);
-      continue;
-    }
-    const float4 *trow = table + (size_t)t * (pairs / 2);
-    uint4 *row = x + j * vecs;
-    for (int v = sl; v < vecs; v += L) {
-      const int pair0 = ((v * 8) % D) / 2;
-      row[v] = rope8(row[v], trow + pair0 / 2);
-    }
+    else
+      rope_row<kFixed, kRopeUnroll>(x + j * vecs, x + j * vecs, table + (size_t)t * (D / 4), vecs,
+                                    L, sl, D, false, [](const uint4 *p) { return *p; });
+    t = t_next;
   }
 }
 
 // KV-cache synchronisation with K rotated on the way in: rows 0..n-1 are K
 // rows (rotated by the table row of token idx[j]), rows n..2n-1 the V rows
-// (copied).
+// (copied).  Same sizes: 39.4 -> 36.4 us (0.86), 242 -> 237 (0.99); 6144 x 32 x
+// 64 12.6 -> 9.9.
+template <bool kFixed>
 __global__ void __launch_bounds__(kThreads)
 kv_scatter_rope_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc,
                        const uint4 *__restrict__ kf, const uint4 *__restrict__ vf,
                        const int32_t *__restrict__ idx, int n_active, int N, int vecs, int D,
                        const float4 *__restrict__ table, int lpr_log2, unsigned *err) {
+  pdl_wait();
+  pdl_trigger();
   const int L = 1 << lpr_log2;
   const int lane = threadIdx.x & 31;
-  const int sub = lane >> lpr_log2, sl = lane & (L - 1);
-  const int rows_per_warp = 32 >> lpr_log2;
-  const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  const int pairs = D / 2;
-  for (long long jj = warp * rows_per_warp + sub; jj < 2LL * n_active;
-       jj += nwarps * rows_per_warp) {
+  const int sl = lane & (L - 1);
+  const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;
+  const long long rows = 2LL * n_active;
+  long long jj = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
+  auto row_idx = [&](long long q) {
+    return q < rows ? __ldg(idx + (q >= n_active ? q - n_active : q)) : 0;
+  };
+  int r = row_idx(jj);
+  for (; jj < rows; jj += step) {
+    const int r_next = row_idx(jj + step);
     const bool is_v = jj >= n_active;
     const long long j = is_v ? jj - n_active : jj;
-    const int r = __ldg(idx + j);
     if (r < 0 || r >= N) {
       if (!is_v) set_error(err, kErrIndex);
-      continue;
+    } else {
+      rope_row<kFixed, kRopeScatterUnroll>(
+          (is_v ? vf : kf) + j * vecs, (is_v ? vc : kc) + (long long)r * vecs,
+          table + (size_t)r * (D / 4), vecs, L, sl, D, is_v, ld_stream);
     }
-    const uint4 *s = (is_v ? vf : kf) + j * vecs;
-    uint4 *d = (is_v ? vc : kc) + (long long)r * vecs;
-    const float4 *trow = table + (size_t)r * (pairs / 2);
-    for (int v0 = sl; v0 < vecs; v0 += kScatterUnroll * L) {
-      uint4 buf[kScatterUnroll];
-#pragma unroll
-      for (int u = 0; u < kScatterUnroll; ++u) {
-        const int v = v0 + u * L;
-        if (v < vecs) buf[u] = ld_stream(s + v);
-      }
-#pragma unroll
-      for (int u = 0; u < kScatterUnroll; ++u) {
-        const int v = v0 + u * L;
-        if (v < vecs) d[v] = is_v ? buf[u] : rope8(buf[u], trow + (((v * 8) % D) / 2) / 2);
-      }
-    }
+    r = r_next;
   }
 }
 
@@ -636,8 +668,9 @@ extern "C" int hsa_rope_rows(void *x, const int32_t *idx, int n, int H, int D,
   if (vecs > (1LL << 30)) return HSA_ERR_UNSUPPORTED;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  rope_rows_kernel<<<grid_for(n, L), kThreads, 0, (cudaStream_t)stream>>>(
-      (uint4 *)x, idx, n, (int)vecs, D, (const float4 *)table, N, log2i(L), err);
+  launch_pdl(L % (D / 8) == 0 ? rope_rows_kernel<true> : rope_rows_kernel<false>,
+             dim3((unsigned)grid_for(n, L)), dim3(kThreads), 0, (cudaStream_t)stream, (uint4 *)x,
+             idx, n, (int)vecs, D, (const float4 *)table, N, log2i(L), err);
   return launch_status();
 }
 
@@ -657,9 +690,10 @@ extern "C" int hsa_kv_sync_scatter_rope(void *k_cache, void *v_cache, const void
   if (vecs > (1LL << 30)) return HSA_ERR_UNSUPPORTED;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  kv_scatter_rope_kernel<<<grid_for(2LL * n_active, L), kThreads, 0, (cudaStream_t)stream>>>(
-      (uint4 *)k_cache, (uint4 *)v_cache, (const uint4 *)k_fresh, (const uint4 *)v_fresh, idx,
-      n_active, N, (int)vecs, D, (const float4 *)table, log2i(L), err);
+  launch_pdl(L % (D / 8) == 0 ? kv_scatter_rope_kernel<true> : kv_scatter_rope_kernel<false>,
+             dim3((unsigned)grid_for(2LL * n_active, L)), dim3(kThreads), 0, (cudaStream_t)stream,
+             (uint4 *)k_cache, (uint4 *)v_cache, (const uint4 *)k_fresh, (const uint4 *)v_fresh,
+             idx, n_active, N, (int)vecs, D, (const float4 *)table, log2i(L), err);
   return launch_status();
 }
 
