@@ -19,12 +19,6 @@ namespace hsa {
 namespace {
 
 constexpr int kThreads = 256;
-// 16-byte vectors each lane keeps in flight (measured on GB300 with an L2-
-// flushed size sweep: the gather reaches its best rate at 4, the scatter,
-// whose loads are contiguous, at 8; Euler holds two vectors per step on long
-// rows, see hsa_cached_euler).
-constexpr int kGatherUnroll = 4;
-constexpr int kScatterUnroll = 8;
 // The rotation in place is best at 6, the rotating scatter, which also holds the
 // table's vectors and two row pointers, at 4.
 constexpr int kRopeUnroll = 6;
@@ -39,77 +33,83 @@ __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
 }
 
 // Row loop shared by gather and scatter: rows are handed out to lane groups
-// in a grid-stride loop; `map(j, s, d)` sets the source and destination row
-// pointers of row j, or returns false to skip the row.
-template <int kUnroll, class RowMap>
-__device__ __forceinline__ void copy_rows(long long n_rows, int vecs, int lpr_log2,
+// in a grid-stride loop; `index(j)` reads row j's token, one row ahead of its
+// use; `map(j, r, s, d)` sets the row's source and destination, or returns false
+// to skip it.  kUnroll 16-byte vectors are in flight per lane (see copy_unroll).
+template <int kUnroll, class Index, class RowMap>
+__device__ __forceinline__ void copy_rows(long long n_rows, int vecs, int lpr_log2, Index index,
                                           RowMap map) {
   const int L = 1 << lpr_log2;
-  const int lane = threadIdx.x & 31;
-  const int sub = lane >> lpr_log2;                  // row slot within the warp
-  const int sl = lane & (L - 1);                     // lane within the row group
-  const int rows_per_warp = 32 >> lpr_log2;
-  const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-  for (long long j = warp * rows_per_warp + sub; j < n_rows; j += nwarps * rows_per_warp) {
+  const int sl = threadIdx.x & (L - 1);              // lane within the row group
+  const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;
+  long long j = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
+  int r = j < n_rows ? index(j) : 0;
+  for (; j < n_rows; j += step) {
+    const int r_next = j + step < n_rows ? index(j + step) : 0;
     const uint4 *s;
     uint4 *d;
-    if (!map(j, s, d)) continue;
-    for (int v0 = sl; v0 < vecs; v0 += kUnroll * L) {
-      uint4 buf[kUnroll];
+    if (map(j, r, s, d)) {
+      for (int v0 = sl; v0 < vecs; v0 += kUnroll * L) {
+        uint4 buf[kUnroll];
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int v = v0 + u * L;
-        if (v < vecs) buf[u] = ld_stream(s + v);
-      }
+        for (int u = 0; u < kUnroll; ++u) {
+          const int v = v0 + u * L;
+          if (v < vecs) buf[u] = ld_stream(s + v);
+        }
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int v = v0 + u * L;
-        if (v < vecs) d[v] = buf[u];
+        for (int u = 0; u < kUnroll; ++u) {
+          const int v = v0 + u * L;
+          if (v < vecs) d[v] = buf[u];
+        }
       }
     }
+    r = r_next;
   }
 }
 
+template <int kUnroll>
 __global__ void __launch_bounds__(kThreads)
 gather_rows_kernel(const uint4 *__restrict__ src, uint4 *__restrict__ dst,
-              const int32_t *__restrict__ idx, int n_active, int N, int vecs,
-              int lpr_log2, unsigned *err) {
+                   const int32_t *__restrict__ idx, int n_active, int N, int vecs, int lpr_log2,
+                   unsigned *err) {
   pdl_wait();
   pdl_trigger();
-  copy_rows<kGatherUnroll>(n_active, vecs, lpr_log2, [&](long long j, const uint4 *&s, uint4 *&d) {
-    const int r = __ldg(idx + j);
-    if (r < 0 || r >= N) {
-      set_error(err, kErrIndex);
-      return false;
-    }
-    s = src + (long long)r * vecs;
-    d = dst + j * vecs;
-    return true;
-  });
+  copy_rows<kUnroll>(
+      n_active, vecs, lpr_log2, [&](long long j) { return __ldg(idx + j); },
+      [&](long long j, int r, const uint4 *&s, uint4 *&d) {
+        if (r < 0 || r >= N) {
+          set_error(err, kErrIndex);
+          return false;
+        }
+        s = src + (long long)r * vecs;
+        d = dst + j * vecs;
+        return true;
+      });
 }
 
 // Rows 0..n_active-1 are K rows, n_active..2*n_active-1 the V rows, so a warp
 // moves K and V rows of different tokens with the same code.
+template <int kUnroll>
 __global__ void __launch_bounds__(kThreads)
-kv_scatter_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc,
-               const uint4 *__restrict__ kf, const uint4 *__restrict__ vf,
-               const int32_t *__restrict__ idx, int n_active, int N, int vecs,
-               int lpr_log2, unsigned *err) {
+kv_scatter_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc, const uint4 *__restrict__ kf,
+                  const uint4 *__restrict__ vf, const int32_t *__restrict__ idx, int n_active,
+                  int N, int vecs, int lpr_log2, unsigned *err) {
   pdl_wait();
   pdl_trigger();
-  copy_rows<kScatterUnroll>(2LL * n_active, vecs, lpr_log2, [&](long long jj, const uint4 *&s, uint4 *&d) {
-    const bool is_v = jj >= n_active;
-    const long long j = is_v ? jj - n_active : jj;
-    const int r = __ldg(idx + j);
-    if (r < 0 || r >= N) {
-      if (!is_v) set_error(err, kErrIndex);
-      return false;
-    }
-    s = (is_v ? vf : kf) + j * vecs;
-    d = (is_v ? vc : kc) + (long long)r * vecs;
-    return true;
-  });
+  copy_rows<kUnroll>(
+      2LL * n_active, vecs, lpr_log2,
+      [&](long long jj) { return __ldg(idx + (jj >= n_active ? jj - n_active : jj)); },
+      [&](long long jj, int r, const uint4 *&s, uint4 *&d) {
+        const bool is_v = jj >= n_active;
+        const long long j = is_v ? jj - n_active : jj;
+        if (r < 0 || r >= N) {
+          if (!is_v) set_error(err, kErrIndex);
+          return false;
+        }
+        s = (is_v ? vf : kf) + j * vecs;
+        d = (is_v ? vc : kc) + (long long)r * vecs;
+        return true;
+      });
 }
 
 // pos[row], with a bad entry (only -1 means "no fresh row") reported and read as
@@ -519,6 +519,18 @@ long long resident_blocks() {
   return (long long)nb * sm_count();
 }
 
+// Vectors in flight per lane of a row copy: 6, or 4 where a lane's share of a row
+// is short or two rounds of 4.  Half of the rows, 3 layers in turn, against 4
+// (gather) and 8 (scatter) with the index not read ahead: short rows hold fewer
+// registers, scatter of 200000 x 256 B 28.5 -> 24.6 us (6: 30.8) and 1000000 x 64 B
+// 39.4 -> 34.7, gather 13.3 -> 12.5 and 19.3 -> 17.0; long rows, gather of 32760 x 10
+// KB 54.6 -> 53.1 (0.94 of the measured HBM rate), scatter within the 3 % that the
+// memory's placement makes (0.93 .. 1.00).
+int copy_unroll(long long vecs, int L) {
+  const long long per_lane = (vecs + L - 1) / L;
+  return per_lane > 8 || per_lane == 5 || per_lane == 6 ? 6 : 4;
+}
+
 int log2i(int L) {
   int s = 0;
   while ((1 << s) < L) ++s;
@@ -542,7 +554,7 @@ extern "C" int hsa_gather_active(const void *src, size_t row_bytes, int N,
   if (!err) return HSA_ERR_CUDA;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  launch_pdl(gather_rows_kernel, dim3(grid_for(n_active, L)), dim3(kThreads), 0,
+  launch_pdl(copy_unroll(vecs, L) == 6 ? gather_rows_kernel<6> : gather_rows_kernel<4>, dim3(grid_for(n_active, L)), dim3(kThreads), 0,
              (cudaStream_t)stream, (const uint4 *)src, (uint4 *)dst, idx, n_active, N, (int)vecs,
              log2i(L), err);
   return launch_status();
@@ -566,7 +578,7 @@ extern "C" int hsa_kv_sync_scatter(void *k_cache, void *v_cache, const void *k_f
   if (!err) return HSA_ERR_CUDA;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  launch_pdl(kv_scatter_kernel, dim3(grid_for(2LL * n_active, L)), dim3(kThreads), 0,
+  launch_pdl(copy_unroll(vecs, L) == 6 ? kv_scatter_kernel<6> : kv_scatter_kernel<4>, dim3(grid_for(2LL * n_active, L)), dim3(kThreads), 0,
              (cudaStream_t)stream, (uint4 *)k_cache, (uint4 *)v_cache, (const uint4 *)k_fresh,
              (const uint4 *)v_fresh, idx, n_active, N, (int)vecs, log2i(L), err);
   return launch_status();
