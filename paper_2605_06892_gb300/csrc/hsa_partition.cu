@@ -74,7 +74,7 @@ __device__ __forceinline__ uint32_t order_key(float f) {
 // keys and tokens stay in L2), so each lets the next one launch at once and
 // what bounds them is latency: every thread issues all its loads before it
 // uses the first, and a tile is shared by 32 warps.  GPU time of a whole
-// partition of 524288 tokens: 281 -> 62 us.
+// partition of 524288 tokens: 281 -> 48 us.
 __global__ void __launch_bounds__(kSortThreads)
 radix_key_kernel(const float *__restrict__ stat, int N, uint32_t *__restrict__ keys,
                  unsigned *err) {
@@ -184,19 +184,31 @@ __global__ void __launch_bounds__(1024) radix_scan_kernel(uint32_t *__restrict__
 
 // Stable scatter of one tile.  Warp w owns tokens [w*128, w*128+128) of the
 // tile and walks them 32 at a time in order; lanes holding the same digit find
-// each other with __match_any_sync, so a token's rank among equal digits in
-// the tile is (earlier warps' count) + (this warp's running count) + (earlier
-// lanes of this step).  vin NULL: the pairs are still in token order.  kout
-// NULL: the last pass, whose keys nothing reads.
+// each other, so a token's rank among equal digits in the tile is (earlier warps'
+// count) + (this warp's running count) + (earlier lanes of this step).  They do so
+// by eight ballots, one per bit: __match_any_sync takes longer the more digits a
+// warp holds, up to 32 on the low digits (9.7 us a pass at 524288 tokens against
+// 7.9); on the last pass, the exponent bits, they are few and it is the faster
+// (5.6 against 6.8).  The tile is first sorted in shared memory, so that
+// neighbouring threads store neighbouring elements of a digit's run (16 on
+// average): stored from where they stood, each 4-byte element cost a 32-byte
+// sector, 12.7 us a pass.  vin NULL: the pairs are
+// still in token order.  kout NULL: the last pass, whose keys nothing reads.
 __global__ void __launch_bounds__(kTileThreads)
 radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict__ vin,
                      uint32_t *__restrict__ kout, int32_t *__restrict__ vout, int N, int shift,
                      const uint32_t *__restrict__ offsets, int tiles) {
   pdl_wait();
   pdl_trigger();
-  __shared__ uint32_t cnt[kTileWarps][256];
+  // the warps' digit counts, then the sorted tile (kTile keys, kTile tokens)
+  __shared__ __align__(16) uint32_t cnt[kTileWarps][256];
+  static_assert(sizeof(cnt) == 2 * kTile * sizeof(uint32_t), "the sorted tile reuses the counts");
+  __shared__ uint32_t base_of[256];                      // digit's first place in the tile
+  __shared__ uint32_t dst_of[256];                       // its first place in the output
+  __shared__ uint32_t warp_sum[8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int base = blockIdx.x * kTile + w * kWarpItems;
+  const int tile0 = blockIdx.x * kTile;
+  const int base = tile0 + w * kWarpItems;
   uint32_t key[kItems];
   int32_t val[kItems];
   uint32_t local[kItems];
@@ -206,6 +218,7 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
     key[it] = n < N ? kin[n] : 0u;
     val[it] = n < N && vin ? vin[n] : n;
   }
+  if (threadIdx.x < 256) dst_of[threadIdx.x] = offsets[threadIdx.x * tiles + blockIdx.x];
   uint4 *c4 = reinterpret_cast<uint4 *>(&cnt[w][0]);
   c4[lane] = make_uint4(0u, 0u, 0u, 0u);                 // this warp's 256 counts
   c4[lane + 32] = make_uint4(0u, 0u, 0u, 0u);
@@ -215,7 +228,18 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
   for (int it = 0; it < kItems; ++it) {
     const bool valid = base + it * 32 + lane < N;
     const uint32_t d = (key[it] >> shift) & 255u;
-    const unsigned peers = __match_any_sync(0xffffffffu, valid ? d : 256u + lane);
+    unsigned peers;
+    if (kout) {
+      peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        const bool bit = d >> b & 1u;
+        const unsigned bal = __ballot_sync(0xffffffffu, bit);
+        peers &= bit ? bal : ~bal;
+      }
+    } else {
+      peers = __match_any_sync(0xffffffffu, valid ? d : 256u + lane);
+    }
     const uint32_t before = valid ? cnt[w][d] : 0u;
     local[it] = before + __popc(peers & lt_mask);
     __syncwarp();
@@ -240,21 +264,58 @@ radix_scatter_kernel(const uint32_t *__restrict__ kin, const int32_t *__restrict
       const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o, 4);
       if (part >= o) incl += t;
     }
-    uint32_t run = offsets[d * tiles + blockIdx.x] + incl - sum;
+    uint32_t run = incl - sum;
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
       cnt[part * kPer + i][d] = run;
       run += c[i];
     }
+    if (part == 3) base_of[d] = run;                     // tokens of the digit in the tile
+  }
+  __syncthreads();
+  // exclusive prefix over digits
+  uint32_t count = 0, incl = 0;
+  if (threadIdx.x < 256) {
+    count = incl = base_of[threadIdx.x];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) warp_sum[w] = incl;
+  }
+  __syncthreads();
+  if (threadIdx.x < 256) {
+    const uint32_t ws = lane < w ? warp_sum[lane & 7] : 0u;   // w < 8: earlier warps only
+    base_of[threadIdx.x] = __reduce_add_sync(0xffffffffu, ws) + incl - count;
   }
   __syncthreads();
 #pragma unroll
   for (int it = 0; it < kItems; ++it) {
+    const uint32_t d = (key[it] >> shift) & 255u;
+    local[it] += base_of[d] + cnt[w][d];
+  }
+  __syncthreads();                                       // the counts have been read
+  uint32_t *skey = &cnt[0][0];
+  int32_t *sval = reinterpret_cast<int32_t *>(skey + kTile);
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
     if (base + it * 32 + lane < N) {
-      const uint32_t d = (key[it] >> shift) & 255u;
-      const uint32_t q = cnt[w][d] + local[it];
-      if (kout) kout[q] = key[it];
-      vout[q] = val[it];
+      skey[local[it]] = key[it];
+      sval[local[it]] = val[it];
+    }
+  }
+  __syncthreads();
+  const int n_tile = min(kTile, N - tile0);
+#pragma unroll
+  for (int it = 0; it < kItems; ++it) {
+    const int i = it * kTileThreads + threadIdx.x;
+    if (i < n_tile) {
+      const uint32_t k = skey[i];
+      const uint32_t d = (k >> shift) & 255u;
+      const uint32_t q = dst_of[d] + (i - base_of[d]);
+      if (kout) kout[q] = k;
+      vout[q] = sval[i];
     }
   }
 }
