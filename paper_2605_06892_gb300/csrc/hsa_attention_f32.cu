@@ -66,8 +66,11 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool vali
                : "memory");
 }
 
+// One block per SM as the stated minimum: without it the compiler holds the
+// 256-thread instances (D = 128) to fewer registers, 8 % slower (16 heads x 128,
+// 2000 queries, 3000 keys: 1350 against 1250 us).
 template <class C>
-__global__ void __launch_bounds__(C::kThreads)
+__global__ void __launch_bounds__(C::kThreads, 1)
 attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
                 const float *__restrict__ kc, const float *__restrict__ vc, int rows1,
                 const float *__restrict__ kb, const float *__restrict__ vb,
