@@ -905,7 +905,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // ------------------------------------------------ softmax / epilogue
     const int t = (warp - 4) >> 2;
     const int wq = warp & 3;                       // TMEM lane quarter of this warp
-    const int r = wq * 32 + lane;                  // row within the Q tile
     const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
     const uint32_t tS = tmem + lane_off + 128 * t;
     const uint32_t tO = tmem + lane_off + C::kOCol0 + D * t;
