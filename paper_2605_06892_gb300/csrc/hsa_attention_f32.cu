@@ -35,7 +35,8 @@ namespace {
 // Measured on GB300 (32 heads x 64, 3072 queries, 6144 keys): 3.03 ms, 51
 // TFLOP/s (the FMA pipe allows 78), against 10.96 ms for one query row per 8
 // threads with scalar shared loads and a shuffle reduction per key; 256 queries
-// x 4 heads x 1024 keys: 22 us against 146 us (64 CTAs, no split of the keys).
+// x 4 heads x 1024 keys: 15.4 us in a graph (64 CTAs without a split of the keys: 146
+// us under ncu).
 template <int D_, int RT_, int WQ_, int WK_>
 struct F32Cfg {
   static constexpr int D = D_, RT = RT_, WQ = WQ_, WK = WK_;

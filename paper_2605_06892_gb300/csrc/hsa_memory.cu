@@ -32,49 +32,64 @@ __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
   return v;
 }
 
-// Row loop shared by gather and scatter: rows are handed out to lane groups
-// in a grid-stride loop; `index(j)` reads row j's token, one row ahead of its
-// use; `map(j, r, s, d)` sets the row's source and destination, or returns false
-// to skip it.  kUnroll 16-byte vectors are in flight per lane (see copy_unroll).
-template <int kUnroll, class Index, class RowMap>
-__device__ __forceinline__ void copy_rows(long long n_rows, int vecs, int lpr_log2, Index index,
-                                          RowMap map) {
-  const int L = 1 << lpr_log2;
-  const int sl = threadIdx.x & (L - 1);              // lane within the row group
-  const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;
-  long long j = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
-  int r = j < n_rows ? index(j) : 0;
-  for (; j < n_rows; j += step) {
-    const int r_next = j + step < n_rows ? index(j + step) : 0;
-    const uint4 *s;
-    uint4 *d;
-    if (map(j, r, s, d)) {
-      for (int v0 = sl; v0 < vecs; v0 += kUnroll * L) {
-        uint4 buf[kUnroll];
+// One row of `vecs` 16-byte vectors by the lanes of a group, kUnroll in flight each.
+template <int kUnroll>
+__device__ __forceinline__ void copy_row(const uint4 *s, uint4 *d, int vecs, int sl, int L) {
+  for (int v0 = sl; v0 < vecs; v0 += kUnroll * L) {
+    uint4 buf[kUnroll];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const int v = v0 + u * L;
-          if (v < vecs) buf[u] = ld_stream(s + v);
-        }
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const int v = v0 + u * L;
-          if (v < vecs) d[v] = buf[u];
-        }
-      }
+    for (int u = 0; u < kUnroll; ++u) {
+      const int v = v0 + u * L;
+      if (v < vecs) buf[u] = ld_stream(s + v);
     }
-    r = r_next;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int v = v0 + u * L;
+      if (v < vecs) d[v] = buf[u];
+    }
   }
 }
 
-template <int kUnroll>
+// Row loop shared by gather and scatter: rows are handed out to lane groups
+// in a grid-stride loop; `index(j)` reads row j's token, with kAhead one row
+// before its use; `map(j, r, s, d)` sets the row's source and destination, or
+// returns false to skip it.  CopyPlan says which form a row length takes.
+template <int kUnroll, bool kAhead, class Index, class RowMap>
+__device__ __forceinline__ void copy_rows(long long n_rows, int vecs, int lpr_log2, Index index,
+                                          RowMap map) {
+  const int L = 1 << lpr_log2;
+  const uint4 *s;
+  uint4 *d;
+  if constexpr (kAhead) {
+    const int sl = threadIdx.x & (L - 1);            // lane within the row group
+    const long long step = ((long long)gridDim.x * blockDim.x) >> lpr_log2;
+    long long j = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lpr_log2;
+    int r = j < n_rows ? index(j) : 0;
+    for (; j < n_rows; j += step) {
+      const int r_next = j + step < n_rows ? index(j + step) : 0;
+      if (map(j, r, s, d)) copy_row<kUnroll>(s, d, vecs, sl, L);
+      r = r_next;
+    }
+  } else {
+    const int lane = threadIdx.x & 31;
+    const int sub = lane >> lpr_log2;                // row slot within the warp
+    const int sl = lane & (L - 1);
+    const int rows_per_warp = 32 >> lpr_log2;
+    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long j = warp * rows_per_warp + sub; j < n_rows; j += nwarps * rows_per_warp)
+      if (map(j, index(j), s, d)) copy_row<kUnroll>(s, d, vecs, sl, L);
+  }
+}
+
+template <int kUnroll, bool kAhead>
 __global__ void __launch_bounds__(kThreads)
 gather_rows_kernel(const uint4 *__restrict__ src, uint4 *__restrict__ dst,
                    const int32_t *__restrict__ idx, int n_active, int N, int vecs, int lpr_log2,
                    unsigned *err) {
   pdl_wait();
   pdl_trigger();
-  copy_rows<kUnroll>(
+  copy_rows<kUnroll, kAhead>(
       n_active, vecs, lpr_log2, [&](long long j) { return __ldg(idx + j); },
       [&](long long j, int r, const uint4 *&s, uint4 *&d) {
         if (r < 0 || r >= N) {
@@ -96,7 +111,7 @@ kv_scatter_kernel(uint4 *__restrict__ kc, uint4 *__restrict__ vc, const uint4 *_
                   int N, int vecs, int lpr_log2, unsigned *err) {
   pdl_wait();
   pdl_trigger();
-  copy_rows<kUnroll>(
+  copy_rows<kUnroll, true>(
       2LL * n_active, vecs, lpr_log2,
       [&](long long jj) { return __ldg(idx + (jj >= n_active ? jj - n_active : jj)); },
       [&](long long jj, int r, const uint4 *&s, uint4 *&d) {
@@ -493,10 +508,10 @@ check_indices_kernel(const int32_t *__restrict__ idx, long long n, int N,
 // Grid for n_rows rows handled by lane groups of size L: up to 8 blocks of
 // 256 threads per SM (a full SM), no more than the rows need; blocks beyond
 // what is resident wait their turn.
-int grid_for(long long n_rows, int L) {
+int grid_for(long long n_rows, int L, int blocks_per_sm = 2048 / kThreads) {
   const long long rows_per_block = (long long)(kThreads / 32) * (32 / L);
   long long blocks = (n_rows + rows_per_block - 1) / rows_per_block;
-  const long long cap = (long long)sm_count() * (2048 / kThreads);
+  const long long cap = (long long)sm_count() * blocks_per_sm;
   if (blocks > cap) blocks = cap;
   return (int)(blocks < 1 ? 1 : blocks);
 }
@@ -519,16 +534,41 @@ long long resident_blocks() {
   return (long long)nb * sm_count();
 }
 
-// Vectors in flight per lane of a row copy: 6, or 4 where a lane's share of a row
-// is short or two rounds of 4.  Half of the rows, 3 layers in turn, against 4
-// (gather) and 8 (scatter) with the index not read ahead: short rows hold fewer
-// registers, scatter of 200000 x 256 B 28.5 -> 24.6 us (6: 30.8) and 1000000 x 64 B
-// 39.4 -> 34.7, gather 13.3 -> 12.5 and 19.3 -> 17.0; long rows, gather of 32760 x 10
-// KB 54.6 -> 53.1 (0.94 of the measured HBM rate), scatter within the 3 % that the
-// memory's placement makes (0.93 .. 1.00).
-int copy_unroll(long long vecs, int L) {
+// How a row copy runs, by the 16-byte vectors each lane moves per row.  Swept over
+// rows of 64 B to 10 KB, 12 to 320 MB (gather also 1 GB), half and all rows, 2 or 3
+// layers in turn, against 4 (gather) and 8 (scatter) vectors in flight, index in
+// place, 8 blocks per SM; ratios are before / now (means: gather 1.05, scatter 1.06;
+// below 1 they are 0.1 to 0.4 us of calls under 10 us, or 1.5 % of 2304-byte rows).
+// Half of 40 x 128 bf16 rows of 32760 tokens, gather and scatter: 160.0 -> 153.0 us.
+//   Grid.  40 to 64 registers leave 4 to 6 blocks of 256 resident; of 8 launched
+//   per SM the rest are an uneven second wave.  32 replace one another as they
+//   end: gather of 1310720 x 256 B 1.13 -> 1.27, scatter of 81920 x 4 KB 1.00 ->
+//   1.06.  The scatter of short rows is as good or better with 8 (163840 x 256 B
+//   1.16 against 1.02): more rows per group hide the index.
+//   Gather.  Up to 2 vectors: 4 in flight, the index one row ahead, 1.00 .. 1.43.
+//   5, 6 or more than 8: 6 in flight take the odd remainder in one round or few,
+//   1.01 .. 1.22 up to 6, 0.96 .. 1.06 above.  3, 4, 7 and 8: 4 with the index in
+//   place, 0.96 .. 1.05 (read ahead it is 0.67 .. 1.0, with 6 0.87 .. 1.05).
+//   Scatter.  4 in flight, index ahead: 1.02 .. 1.40 up to 2 vectors, 0.98 .. 1.20
+//   above; a fifth vector that is not whole takes 6 (129 vectors: 1.00 .. 1.02
+//   against 0.89 .. 0.99).
+struct CopyPlan {
+  int unroll;
+  bool ahead;
+  int blocks;      // per SM, at most
+};
+
+CopyPlan gather_plan(long long vecs, int L) {
   const long long per_lane = (vecs + L - 1) / L;
-  return per_lane > 8 || per_lane == 5 || per_lane == 6 ? 6 : 4;
+  if (per_lane <= 2) return CopyPlan{4, true, 32};
+  if (per_lane > 8 || per_lane == 5 || per_lane == 6) return CopyPlan{6, true, 32};
+  return CopyPlan{4, false, 32};
+}
+
+CopyPlan scatter_plan(long long vecs, int L) {
+  const long long per_lane = (vecs + L - 1) / L;
+  if (per_lane == 5 && vecs % L != 0) return CopyPlan{6, true, 8};
+  return CopyPlan{4, true, per_lane <= 2 ? 8 : 32};
 }
 
 int log2i(int L) {
@@ -554,8 +594,12 @@ extern "C" int hsa_gather_active(const void *src, size_t row_bytes, int N,
   if (!err) return HSA_ERR_CUDA;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  launch_pdl(copy_unroll(vecs, L) == 6 ? gather_rows_kernel<6> : gather_rows_kernel<4>, dim3(grid_for(n_active, L)), dim3(kThreads), 0,
-             (cudaStream_t)stream, (const uint4 *)src, (uint4 *)dst, idx, n_active, N, (int)vecs,
+  const CopyPlan plan = gather_plan(vecs, L);
+  launch_pdl(plan.unroll == 6 ? gather_rows_kernel<6, true>
+             : plan.ahead     ? gather_rows_kernel<4, true>
+                              : gather_rows_kernel<4, false>,
+             dim3(grid_for(n_active, L, plan.blocks)), dim3(kThreads), 0, (cudaStream_t)stream,
+             (const uint4 *)src, (uint4 *)dst, idx, n_active, N, (int)vecs,
              log2i(L), err);
   return launch_status();
 }
@@ -578,7 +622,9 @@ extern "C" int hsa_kv_sync_scatter(void *k_cache, void *v_cache, const void *k_f
   if (!err) return HSA_ERR_CUDA;
   const int L = lanes_per_row(vecs);
   count_launches(1);
-  launch_pdl(copy_unroll(vecs, L) == 6 ? kv_scatter_kernel<6> : kv_scatter_kernel<4>, dim3(grid_for(2LL * n_active, L)), dim3(kThreads), 0,
+  const CopyPlan plan = scatter_plan(vecs, L);
+  launch_pdl(plan.unroll == 6 ? kv_scatter_kernel<6> : kv_scatter_kernel<4>,
+             dim3(grid_for(2LL * n_active, L, plan.blocks)), dim3(kThreads), 0,
              (cudaStream_t)stream, (uint4 *)k_cache, (uint4 *)v_cache, (const uint4 *)k_fresh,
              (const uint4 *)v_fresh, idx, n_active, N, (int)vecs, log2i(L), err);
   return launch_status();
