@@ -89,6 +89,7 @@ _SIGS = {
 }
 
 _lib = None
+# torch's own, not part of its public interface: None where a torch lacks them
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 _current_device = getattr(torch._C, "_cuda_getDevice", None)
 
@@ -125,9 +126,9 @@ def _stream(stream):
     if stream is None:
         # The current stream's handle as torch keeps it: 0.2 us, against 2.9 us
         # for building the torch.cuda.Stream object (a third of a small call's
-        # host time on the Grace host).  Before CUDA is initialised the object's
-        # constructor initialises it.
-        if torch.cuda.is_initialized():
+        # host time on the Grace host).  Before CUDA is initialised, and on a torch
+        # without these two functions, the object's constructor serves.
+        if _raw_stream and _current_device and torch.cuda.is_initialized():
             return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
