@@ -28,6 +28,7 @@ __all__ = [
     "hsa_active_attention_workspace_bytes",
     "hsa_cached_euler", "hsa_cached_euler_l1rel",
     "hsa_get_device_error", "hsa_launch_count", "hsa_test_inject_attention_stall",
+    "hsa_test_f32_cluster",
 ]
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -86,6 +87,7 @@ _SIGS = {
     "hsa_get_device_error": ([_c_p], _c_int),
     "hsa_launch_count": ([], ctypes.c_ulonglong),
     "hsa_test_inject_attention_stall": ([_c_int], _c_int),
+    "hsa_test_f32_cluster": ([_c_int] * 7, _c_int),
 }
 
 _lib = None
@@ -356,3 +358,12 @@ def hsa_test_inject_attention_stall(mode: int) -> int:
     launches never load their first value tile, so the bounded wait for it runs
     out and HSA_ERR_TIMEOUT is reported; mode 0 restores normal operation."""
     return _check(lib().hsa_test_inject_attention_stall(mode), "hsa_test_inject_attention_stall")
+
+
+def hsa_test_f32_cluster(n_active: int, N: int, H: int, D: int, sms: int, wide_most: int,
+                         deep_most: int) -> int:
+    """Test hook (include/hsa_test.h): CTAs per cluster of the fp32 attention's launch
+    plan where clusters of at most wide_most / deep_most CTAs can be resident, plus
+    256 for its deep kernel.  Needs no GPU."""
+    return _check(lib().hsa_test_f32_cluster(n_active, N, H, D, sms, wide_most, deep_most),
+                  "hsa_test_f32_cluster")

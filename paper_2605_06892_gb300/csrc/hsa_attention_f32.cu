@@ -6,6 +6,7 @@
 
 #include "hsa_internal.cuh"
 #include "hsa_ptx.cuh"
+#include "hsa_test.h"
 
 namespace hsa {
 namespace {
@@ -348,23 +349,26 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
 // the deep one (32 rows, the CTA's warps on different keys), and how many CTAs
 // of a cluster split the keys.  Both run 4 or 8 warps on the same tile code, so
 // the time of a plan is the CTAs per SM times the stages each runs (plus about
-// half a stage for the query load and the merge); the smallest wins.
+// half a stage for the query load and the merge); the smallest wins.  A cluster
+// has no more CTAs than can be resident (`wide_most`, `deep_most`; a slice of the
+// GPU may hold fewer than 8 together): a larger one would not launch.
 struct F32Plan {
   bool deep;
   int splits;
 };
 
 template <class Wide, class Deep>
-F32Plan f32_plan(int n_active, int N, int H, int sms) {
+F32Plan f32_plan(int n_active, int N, int H, int sms, int wide_most, int deep_most) {
   F32Plan best{false, 1};
   double best_cost = 0.0;
   for (int deep = 0; deep < 2; ++deep) {
     const int rows = deep ? Deep::kRows : Wide::kRows, keys = deep ? Deep::kKeys : Wide::kKeys;
     const int threads = deep ? Deep::kThreads : Wide::kThreads;
+    const int most = deep ? deep_most : wide_most;
     const long long stages = ((long long)N + keys - 1) / keys;
     const long long units = ((long long)n_active + rows - 1) / rows * H;
     for (int splits = 1; splits <= 8; splits *= 2) {
-      if (splits > 1 && stages < splits) break;
+      if (splits > 1 && (stages < splits || splits > most)) break;
       const long long per_sm = (units * splits + sms - 1) / sms;
       const double cost = (double)per_sm * threads *
                           ((double)((stages + splits - 1) / splits) + (splits > 1 ? 0.6 : 0.5));
@@ -377,20 +381,52 @@ F32Plan f32_plan(int n_active, int N, int H, int sms) {
   return best;
 }
 
+// D = 64: 8 rows per lane (64 accumulators of O); D = 128: 4, for the same count.
+template <int D>
+using F32Wide = F32Cfg<D, D == 64 ? 8 : 4, D == 64 ? 4 : 8, 1>;
+template <int D>
+using F32Deep = F32Cfg<D, D == 64 ? 8 : 4, D == 64 ? 1 : 2, D == 64 ? 4 : 2>;
+
+// Opts kernel C in to its shared memory on the current device; returns the CTAs of
+// the largest cluster (8, 4, 2 or 1) of which one can be resident, 0 on failure.
+// Resolved once per device.
+template <class C>
+int f32_cluster_most() {
+  static std::atomic<int> most[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int n = most[dev].load();
+  if (n) return n;
+  if (cudaFuncSetAttribute(attn_f32_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           C::kSmem) != cudaSuccess)
+    return 0;
+  for (n = 8; n > 1; n /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n);
+    cfg.blockDim = dim3(C::kThreads);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)n;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, attn_f32_kernel<C>, &cfg) == cudaSuccess &&
+        clusters >= 1)
+      break;
+  }
+  cudaGetLastError();                          // a refused query leaves no sticky error
+  most[dev].store(n);
+  return n;
+}
+
 template <class C>
 int launch_f32_cfg(int splits, const float *q, const int32_t *q_idx, int n_active,
                    const float *k_cache, const float *v_cache, int rows1, const float *k_base,
                    const float *v_base, int N, int H, float scale, float *out,
                    cudaStream_t stream, unsigned *err) {
-  static std::atomic<int> configured[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HSA_ERR_CUDA;
-  if (!configured[dev].load()) {
-    if (cudaFuncSetAttribute(attn_f32_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::kSmem) != cudaSuccess)
-      return HSA_ERR_CUDA;
-    configured[dev].store(1);
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((n_active + (long long)C::kRows - 1) / C::kRows * splits), H);
   cfg.blockDim = dim3(C::kThreads);
@@ -416,11 +452,12 @@ template <int D>
 int launch_f32(const void *q, const int32_t *q_idx, int n_active, const void *k_cache,
                const void *v_cache, int rows1, const void *k_base, const void *v_base, int rows2,
                int H, float scale, void *out, cudaStream_t stream, unsigned *err) {
-  // D = 64: 8 rows per lane (64 accumulators of O); D = 128: 4, for the same count.
-  using Wide = F32Cfg<D, D == 64 ? 8 : 4, D == 64 ? 4 : 8, 1>;
-  using Deep = F32Cfg<D, D == 64 ? 8 : 4, D == 64 ? 1 : 2, D == 64 ? 4 : 2>;
+  using Wide = F32Wide<D>;
+  using Deep = F32Deep<D>;
   const int N = rows1 + rows2;
-  const F32Plan plan = f32_plan<Wide, Deep>(n_active, N, H, sm_count());
+  const int wide_most = f32_cluster_most<Wide>(), deep_most = f32_cluster_most<Deep>();
+  if (!wide_most || !deep_most) return HSA_ERR_CUDA;
+  const F32Plan plan = f32_plan<Wide, Deep>(n_active, N, H, sm_count(), wide_most, deep_most);
   auto f = [](const void *p) { return static_cast<const float *>(p); };
   return plan.deep
              ? launch_f32_cfg<Deep>(plan.splits, f(q), q_idx, n_active, f(k_cache), f(v_cache),
@@ -444,3 +481,15 @@ int launch_attention_f32(const void *q, const int32_t *q_idx, int n_active, cons
 }
 
 }  // namespace hsa
+
+extern "C" int hsa_test_f32_cluster(int n_active, int N, int H, int D, int sms, int wide_most,
+                                    int deep_most) {
+  using namespace hsa;
+  if (n_active < 1 || N < 1 || H < 1 || sms < 1 || wide_most < 1 || deep_most < 1 ||
+      (D != 64 && D != 128))
+    return HSA_ERR_INVALID_ARG;
+  const F32Plan p =
+      D == 128 ? f32_plan<F32Wide<128>, F32Deep<128>>(n_active, N, H, sms, wide_most, deep_most)
+               : f32_plan<F32Wide<64>, F32Deep<64>>(n_active, N, H, sms, wide_most, deep_most);
+  return p.deep ? 256 + p.splits : p.splits;
+}
