@@ -783,7 +783,7 @@ extern "C" int hsa_check_indices(const int32_t *idx, int n, int N, void *workspa
   if (!err) return HSA_ERR_CUDA;
   const long long cap = (long long)sm_count() * (2048 / kThreads);
   const long long n_vec = (long long)(need / 16);
-  long long b0 = (n_vec + kThreads - 1) / kThreads, b1 = (n + kThreads - 1) / kThreads;
+  long long b0 = (n_vec + kThreads - 1) / kThreads, b1 = ((long long)n + kThreads - 1) / kThreads;
   b0 = b0 < 1 ? 1 : (b0 > cap ? cap : b0);
   b1 = b1 > cap ? cap : b1;
   cudaStream_t s = (cudaStream_t)stream;

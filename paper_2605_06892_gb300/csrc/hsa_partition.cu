@@ -53,7 +53,7 @@ struct SortLayout {
 // scratch array of hsa_partition_static is sized by this same formula.
 constexpr SortLayout sort_layout(int N) {
   SortLayout L{};
-  L.tiles = (N + kTile - 1) / kTile;
+  L.tiles = (int)(((long long)N + kTile - 1) / kTile);
   const size_t a = align256((size_t)N * 4);
   L.keys0 = 0;
   L.keys1 = a;
@@ -81,7 +81,7 @@ radix_key_kernel(const float *__restrict__ stat, int N, uint32_t *__restrict__ k
   pdl_wait();
   pdl_trigger();
   const bool vec = (reinterpret_cast<uintptr_t>(stat) & 15) == 0;
-  const int n4 = (N + 3) >> 2;
+  const int n4 = (int)(((unsigned)N + 3u) >> 2);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gridDim.x * blockDim.x) {
     float f[4];
     if (vec && 4 * i + 3 < N) {
@@ -792,7 +792,10 @@ group_assign_kernel(const int32_t *__restrict__ sorted_tokens, int N, int K, Gro
                     int32_t *__restrict__ group_of) {
   pdl_wait();
   pdl_trigger();
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < N; r += gridDim.x * blockDim.x) {
+  // unsigned: the index one stride past the last token may pass 2^31
+  for (unsigned u = blockIdx.x * blockDim.x + threadIdx.x; u < (unsigned)N;
+       u += gridDim.x * blockDim.x) {
+    const int r = (int)u;
     const int token = sorted_tokens[r];
     int g = 0;
     for (int k = 0; k < K; ++k)
@@ -1097,7 +1100,7 @@ extern "C" int hsa_partition(const float *stat, int N, int T, const int *budgets
   }
   // The scan's cluster is one CTA where a cluster of 8 cannot be resident.
   const unsigned scan_ctas = cluster_scan_ready() ? kScanCtas : 1;
-  const int ew_blocks = (int)std::min<long long>((N + kSortThreads - 1) / kSortThreads,
+  const int ew_blocks = (int)std::min<long long>(((long long)N + kSortThreads - 1) / kSortThreads,
                                                  (long long)sm_count() * 8);
   count_launches(1);
   launch_pdl(radix_key_kernel, dim3((ew_blocks + 3) / 4), dim3(kSortThreads), 0, s, stat, N,
@@ -1154,12 +1157,13 @@ extern "C" int hsa_partition_active(const int32_t *group_of, int N, int T, const
 // rank into the baseline group.
 
 __global__ void uniform_stat_kernel(float *__restrict__ stat, int N) {
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x)
-    stat[n] = (float)(((uint32_t)(n + 1) * 2654435769u) >> 8);
+  for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < (unsigned)N;
+       n += gridDim.x * blockDim.x)
+    stat[n] = (float)(((n + 1) * 2654435769u) >> 8);
 }
 
 __global__ void reserve_frame_kernel(float *__restrict__ stat, int frame_tokens) {
-  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < frame_tokens;
+  for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < (unsigned)frame_tokens;
        n += gridDim.x * blockDim.x)
     stat[n] = 3.40282347e38f;
 }
@@ -1218,7 +1222,7 @@ extern "C" int hsa_uniform_stat(float *stat, int N, hsa_stream_t stream) {
   if (N < 0) return HSA_ERR_INVALID_ARG;
   if (N == 0) return HSA_OK;
   if (!stat) return HSA_ERR_INVALID_ARG;
-  const int blocks = (int)std::min<long long>((N + 255) / 256, (long long)sm_count() * 8);
+  const int blocks = (int)std::min<long long>(((long long)N + 255) / 256, (long long)sm_count() * 8);
   count_launches(1);
   uniform_stat_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(stat, N);
   return launch_status();
@@ -1229,7 +1233,8 @@ extern "C" int hsa_reserve_first_frame(float *stat, int N, int frame_tokens,
   if (N < 0 || frame_tokens < 0 || frame_tokens > N) return HSA_ERR_INVALID_ARG;
   if (frame_tokens == 0) return HSA_OK;
   if (!stat) return HSA_ERR_INVALID_ARG;
-  const int blocks = (int)std::min<long long>((frame_tokens + 255) / 256, (long long)sm_count() * 8);
+  const int blocks = (int)std::min<long long>(((long long)frame_tokens + 255) / 256,
+                                               (long long)sm_count() * 8);
   count_launches(1);
   reserve_frame_kernel<<<blocks, 256, 0, (cudaStream_t)stream>>>(stat, frame_tokens);
   return launch_status();
