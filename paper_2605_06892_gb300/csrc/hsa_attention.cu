@@ -578,20 +578,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  // Launched with programmatic dependent launch: up to here the block touches
+  // only its own shared memory, and runs beside the end of the kernel before it;
+  // wait for that kernel and those before it (the KV scatter writes the keys read
+  // below).  TMEM is taken after the wait, never before: a block that held it while
+  // waiting could keep it from a block of that kernel (another library's, which lets
+  // its dependents start before it allocates) on the same SM, and each would wait
+  // for the other.  For the same reason the next kernel may start only once this
+  // block has its own.  The blocks of the last wave let it start launching onto the
+  // SMs they free; no block of this grid is still waiting for an SM by then.
+  pdl_wait();
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_addr(&tmem_base_sh)),
                  "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (blockIdx.x + (unsigned)a.wave >= gridDim.x) pdl_trigger();
   }
-  // Launched with programmatic dependent launch: up to here the block touches
-  // only its own SM, and runs beside the end of the kernel before it; wait for
-  // that kernel and those before it (the KV scatter writes the keys read below).
-  // The blocks of the last wave let the next kernel start launching onto the SMs
-  // they free; no block of this grid is still waiting for an SM by then.
-  pdl_wait();
-  if (blockIdx.x + (unsigned)a.wave >= gridDim.x) pdl_trigger();
   // The first key tiles load while the CTA loads its query rows below, and no
   // more than the first MMAs need: a whole ring's worth on every SM at once held
   // the query rows up for 2000 clocks.
