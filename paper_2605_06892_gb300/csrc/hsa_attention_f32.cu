@@ -31,13 +31,22 @@ namespace {
 //            memory, so small layers fill the GPU in one launch, without a
 //            workspace.
 // The softmax reference of a row moves only when a score passes it by more
-// than 2^8 (exact whatever the reference: the final division removes it), so
-// most tiles need no reduction across lanes and no rescale of O.
-// Measured on GB300 (32 heads x 64, 3072 queries, 6144 keys): 3.03 ms, 51
+// than 2^kLag (exact whatever the reference: the final division removes it), so
+// most tiles need no reduction across lanes and no rescale of O.  The p that O is
+// formed with are at most 1 all the same (times 2^-kLag, exact, given back by the
+// division), so that large values of V overflow no sooner than with the row's
+// maximum as the reference: 0.6 % at D = 64, 0.2 % at D = 128, the same bits.  (The
+// row's sum scaled too: 1.0 %; the reference set 2^kLag above the maximum costs no
+// time, but the exponents' larger arguments round more coarsely, error + 3 to 18 %; a
+// second pass over the keys after an O that is not finite spills, 2 to 9 %.)
+// Measured on GB300 (32 heads x 64, 3072 queries, 6144 keys): 3.05 ms, 51
 // TFLOP/s (the FMA pipe allows 78), against 10.96 ms for one query row per 8
 // threads with scalar shared loads and a shuffle reduction per key; 256 queries
 // x 4 heads x 1024 keys: 15.4 us in a graph (64 CTAs without a split of the keys: 146
 // us under ncu).
+constexpr float kLag = 8.f;                        // log2 units
+constexpr float kLagFactor = 256.f;                // 2^kLag
+
 template <int D_, int RT_, int WQ_, int WK_>
 struct F32Cfg {
   static constexpr int D = D_, RT = RT_, WQ = WQ_, WK = WK_;
@@ -51,7 +60,7 @@ struct F32Cfg {
   static constexpr int kQFloats = kRows * kQStride;
   static constexpr int kPFloats = 32 * kPStride;            // per warp
   // After the key loop the same memory holds the partial results: O
-  // [WK][kRows][D], then (m, l) [WK][kRows], then the merge weights and 1/l.
+  // [WK][kRows][D], then (m, l) [WK][kRows], then the merge weights and 2^kLag / l.
   static constexpr int kPartO = WK * kRows * D;
   static constexpr int kPartML = 2 * WK * kRows;
   static constexpr int kMerge = 8 * WK * kRows + kRows;
@@ -160,6 +169,7 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
 #pragma unroll
     for (int d = 0; d < 2 * kDV; ++d) o2[i][d] = 0ull;
   }
+  constexpr float kPScale = 1.f / kLagFactor;
   const float *qrow = sQ + (wq * C::kWarpRows + rg) * C::kQStride;
   for (int g = g0; g < g1; ++g) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -207,7 +217,7 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
       const float mx = fmaxf(max3f(s[i][0], s[i][1], s[i][2]), s[i][3]);
-      move |= fmaf(mx, scale_log2, -m[i]) > 8.f;
+      move |= fmaf(mx, scale_log2, -m[i]) > kLag;
     }
     if (__any_sync(0xffffffffu, move)) {
 #pragma unroll
@@ -236,7 +246,7 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
         l2[i / 2] = add2(l2[i / 2], pack2(__float_as_uint(p[0]), __float_as_uint(p[1])));
         l2[i / 2 + 1] = add2(l2[i / 2 + 1], pack2(__float_as_uint(p[2]), __float_as_uint(p[3])));
         *reinterpret_cast<float4 *>(sP + (cl + 8 * j) * C::kPStride + (i + rg) * 4) =
-            make_float4(p[0], p[1], p[2], p[3]);
+            make_float4(p[0] * kPScale, p[1] * kPScale, p[2] * kPScale, p[3] * kPScale);
       }
     }
     __syncwarp();
@@ -276,7 +286,7 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
     for (int i = 0; i < RT; ++i) {
       const int j = row0 + wq * C::kWarpRows + rg + 4 * i;
       if (j >= n_active) continue;
-      const float inv = 1.f / l[i];
+      const float inv = kLagFactor / l[i];
       float *dst = out + ((size_t)j * H + h) * D + 4 * cl;
 #pragma unroll
       for (int d = 0; d < kDV; ++d)
@@ -318,7 +328,7 @@ attn_f32_kernel(const float *__restrict__ q, const int32_t *__restrict__ q_idx,
       pW[p * C::kRows + threadIdx.x] = w;
       L = fmaf(w, v.y, L);
     }
-    pInv[threadIdx.x] = 1.f / L;
+    pInv[threadIdx.x] = kLagFactor / L;
   }
   __syncthreads();
   for (int e = threadIdx.x; e < rows * (D / 4); e += C::kThreads) {
