@@ -477,6 +477,8 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
   __shared__ int slot[kMaxBounds];                     // first boundary with the same range
   __shared__ int target[kMaxBounds];                   // boundary's rank; -1: 0 or N
   __shared__ int split;                                // whether a range holds too many keys
+  __shared__ int whole;                                // whether a pass left one's keys together
+  __shared__ uint32_t kmn[kMaxBounds], kmx[kMaxBounds];   // such a range's keys in this CTA
   __shared__ unsigned long long thr[kMaxBounds];       // boundary pair (key << 32 | token)
   __shared__ int eqc[kMaxBounds];                      // local keys equal to a boundary key
   __shared__ int warp_tot[kCsThreads / 32];
@@ -520,7 +522,7 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
     count[threadIdx.x] = 0;
     fill[threadIdx.x] = kCsList;
   }
-  if (threadIdx.x == 0) split = 0;
+  if (threadIdx.x == 0) split = whole = 0;
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   kmax = __reduce_max_sync(0xffffffffu, kmax);
   if (lane == 0) {
@@ -601,9 +603,15 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
   }
   __syncthreads();
   // Split the ranges that hold too many keys, 256 ways at a time.  All of them
-  // are 2^s wide here, and every thread of the cluster takes the same turns.
+  // are 2^s wide here, and every thread of the cluster takes the same turns.  A pass
+  // that leaves all keys of a range together may have met a value that fills it (a
+  // statistic of few values), so the next one also looks at the keys' extremes and
+  // need not split down to that value: 8 values, 4865 tokens 23.2 -> 17.6 us (18.6 by
+  // ranking), 75600 38.6 -> 31.1.  Looking in every pass would be better for them (13.0,
+  // 23.5) but costs spread statistics 3 to 13 %, after such a pass only 0 to 0.3 us.
   while (__builtin_expect(split, 0)) {
     const int ns = max(0, s - 8);
+    const bool look = whole;
     if (threadIdx.x < nb) {
       const int j = threadIdx.x;
       int first = -1;
@@ -614,18 +622,46 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
       slot[j] = first;                                 // -1: not split
     }
     cl.sync();                  // every CTA has read the histograms of the last pass
-    if (threadIdx.x == 0) split = 0;
+    if (threadIdx.x == 0) split = whole = 0;
+    if (look && threadIdx.x < nb) {
+      kmn[threadIdx.x] = 0xffffffffu;
+      kmx[threadIdx.x] = 0u;
+    }
     for (int i = threadIdx.x; i < nb * 256; i += kCsThreads) hist[i] = 0u;
     __syncthreads();
-    for (int i = threadIdx.x; i < n_loc; i += kCsThreads) {
-      const uint32_t k = skey[i];
-      for (int j = 0; j < nb; ++j)
-        if (slot[j] == j && (k - low[j]) >> s == 0)
+    if (__builtin_expect(look, 0)) {
+      for (int i = threadIdx.x; i < n_loc; i += kCsThreads) {
+        const uint32_t k = skey[i];
+        for (int j = 0; j < nb; ++j) {
+          if (slot[j] != j || (k - low[j]) >> s != 0) continue;
           atomicAdd(&hist[j * 256 + ((k - low[j]) >> ns)], 1u);
+          if (k < kmn[j]) atomicMin(&kmn[j], k);
+          if (k > kmx[j]) atomicMax(&kmx[j], k);
+        }
+      }
+    } else {
+      for (int i = threadIdx.x; i < n_loc; i += kCsThreads) {
+        const uint32_t k = skey[i];
+        for (int j = 0; j < nb; ++j)
+          if (slot[j] == j && (k - low[j]) >> s == 0)
+            atomicAdd(&hist[j * 256 + ((k - low[j]) >> ns)], 1u);
+      }
     }
     cl.sync();                                         // every CTA's histograms are complete
     // warp j picks boundary j's part of its range
-    if (w < nb && slot[w] >= 0) {
+    uint32_t mn = 1u, mx = 0u;
+    if (look && w < nb && slot[w] >= 0) {
+      mn = *cl.map_shared_rank(&kmn[slot[w]], lane % kCsCtas);
+      mx = *cl.map_shared_rank(&kmx[slot[w]], lane % kCsCtas);
+      mn = __reduce_min_sync(0xffffffffu, mn);
+      mx = __reduce_max_sync(0xffffffffu, mx);
+    }
+    if (mn == mx) {                                    // one value: low, and done
+      if (lane == 0) {
+        low[w] = mn;
+        sh[w] = 0;
+      }
+    } else if (w < nb && slot[w] >= 0) {
       const int t = target[w] - below[w];              // rank among the range's keys
       int c[8], before[8], sum = 0;
 #pragma unroll
@@ -659,6 +695,7 @@ cluster_select_kernel(const float *__restrict__ stat, int N, int chunk, int K, G
             low[w] += (uint32_t)(8 * lane + d) << ns;
             sh[w] = ns;
             below[w] = target[w] - at;
+            if (c[d] == count[w]) whole = 1;
             count[w] = c[d];
             fill[w] = before[d];
             if (c[d] > kCsList && ns > 0) split = 1;
