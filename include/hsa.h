@@ -176,6 +176,7 @@ int hsa_reserve_first_frame(float *stat, int N, int frame_tokens, hsa_stream_t s
  *   where      device, int32 [N] or NULL, written (old -> new); undo the
  *              reordering with hsa_gather_active(.., where, N, ..).
  *   group_new  device, int32 [N] or NULL, written: group_of[order[r]].
+ * None of the three may overlap group_of.
  * A group_of that disagrees with n_baseline is reported as HSA_ERR_INDEX. */
 int hsa_reorder_tokens(const int32_t *group_of, int N, int n_baseline, int32_t *order,
                        int32_t *where, int32_t *group_new, hsa_stream_t stream);
@@ -188,6 +189,7 @@ int hsa_reorder_tokens(const int32_t *group_of, int N, int n_baseline, int32_t *
  *   group_of  device, int32 [N] in [0, K).
  *   idx       device, int32 [>= |A_i|], written: active token ids ascending.
  *   pos       device, int32 [N] or NULL, written: rank of n in idx, or -1.
+ * idx and pos must not overlap group_of.
  * |A_i| is hsa_active_count(...) of the same groups, known on the host.  A
  * group id outside [0, K) is reported as HSA_ERR_INDEX (that token is then
  * treated as skipped). */

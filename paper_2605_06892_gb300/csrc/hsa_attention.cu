@@ -883,7 +883,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       // phase too; a named barrier takes a tenth of that.  So this warp makes
       // the (bounded) test, ahead of need where the scores are computed ahead,
       // and meets the softmax group.  It meets even after a failed wait.  24 x
-      // 64, N = 32760: 1508 -> 1595 TFLOP/s; Wan-1.3B shape 2005 -> 2027.
+      // 64, N = 32760: 1508 -> 1595 TFLOP/s; D = 128 within its spread.
       bool live = true;
       for (int j = 0; j < nT; ++j) {
 #pragma unroll

@@ -424,7 +424,7 @@ __device__ __forceinline__ void rope_row(const uint4 *s, uint4 *d, const float4 
 // row; the index of its next row is loaded one row ahead.  HBM-bound; half of the
 // tokens, 3 layers in turn, against one vector in flight per lane and a remainder
 // by D for each: 32760 tokens x 12 x 128 24.8 -> 18.5 us (0.88 of the measured HBM
-// rate), 75600 x 40 x 128 158 -> 120 (0.99).
+// rate), 75600 x 40 x 128 158 -> 117.7 (1.01).
 template <bool kFixed>
 __global__ void __launch_bounds__(kThreads)
 rope_rows_kernel(uint4 *__restrict__ x, const int32_t *__restrict__ idx, int n, int vecs, int D,
@@ -450,7 +450,7 @@ rope_rows_kernel(uint4 *__restrict__ x, const int32_t *__restrict__ idx, int n, 
 
 // KV-cache synchronisation with K rotated on the way in: rows 0..n-1 are K
 // rows (rotated by the table row of token idx[j]), rows n..2n-1 the V rows
-// (copied).  Same sizes: 39.4 -> 36.4 us (0.86), 242 -> 237 (0.99); 6144 x 32 x
+// (copied).  Same sizes: 39.4 -> 36.4 us (0.86), 242 -> 232 (1.01); 6144 x 32 x
 // 64 12.6 -> 9.9.
 template <bool kFixed>
 __global__ void __launch_bounds__(kThreads)
